@@ -15,6 +15,7 @@
 
 #include "../../include/rihf.h"
 #include "common.cuh"
+#include "eri3_lane.cuh"
 #include "integrals.cuh"
 #include "jk.cuh"
 #include "linalg.cuh"
@@ -494,7 +495,11 @@ struct rihf_ctx {
   int* d_ticket = nullptr;  // their ticket counter (zero between launches)
   ShellPair* d_pairs = nullptr;
   int2* d_tasks = nullptr;           // (pair, auxiliary shell) tasks, grouped by shared-memory class
-  TaskGroup groups[kTaskGroups];
+  TaskGroup groups[kTaskGroups];     // Cartesian basis: warp-cooperative kernels (integrals.cu)
+  LaneTasks lane;                    // spherical basis: one lane per task (eri3_lane.cuh)
+  LaneChunk* d_chunks = nullptr;     // its chunk lists
+  size_t chunk_cap = 0;
+  KetTable* d_ket = nullptr;
   double* d_schwarz = nullptr;
   bool schwarz_ok = false;
   bool schwarz_fresh = false;   // d_schwarz holds Q of the current geometry
@@ -678,6 +683,33 @@ static const std::vector<double>& boys_host() {
 // Rebuild the class-grouped 3-centre task lists from the current pair list.
 static void refresh_tasks(rihf_ctx* c) {
   upload(c->d_pp_off, pair_prim_offsets(c->pairs_h, c->hp.nprim), c->stream);
+  if (c->opt.pure) {
+    // spherical auxiliary functions: the harmonic ket recursion, one lane per task
+    std::vector<int2> list;
+    std::vector<LaneChunk> chunks[kLaneGroups];
+    lane_flops(c->pairs_h, c->hp.l, c->hp.nprim, c->hp.atom, c->ha.l, c->ha.nprim, c->ha.atom,
+               build_ket_tables(c->tr_h, c->nf_h), &c->flops_eri3, &c->flops_grad3);
+    build_lane_tasks(c->pairs_h, c->hp.l, c->hp.atom, c->ha.l, c->ha.atom, c->sms, list, chunks);
+    upload(c->d_tasks, list, c->stream);
+    size_t n = 0;
+    for (const auto& v : chunks) n += v.size();
+    if (n > c->chunk_cap) {
+      if (c->d_chunks) cudaFree(c->d_chunks);
+      c->d_chunks = nullptr;
+      c->lane = LaneTasks();
+      c->d_chunks = dalloc<LaneChunk>(n);
+      c->chunk_cap = n;
+    }
+    size_t at = 0;
+    for (int g = 0; g < kLaneGroups; ++g) {
+      c->lane.chunks[g] = c->d_chunks + at;
+      c->lane.nchunk[g] = (long long)chunks[g].size();
+      upload(c->d_chunks + at, chunks[g], c->stream);
+      at += chunks[g].size();
+    }
+    RIHF_CUDA(cudaStreamSynchronize(c->stream));   // the host lists are temporaries
+    return;
+  }
   std::vector<std::vector<int2>> tasks;
   std::vector<int> se, sg;
   // largest primitive exponent per primary shell, smallest per auxiliary shell
@@ -688,9 +720,9 @@ static void refresh_tasks(rihf_ctx* c) {
     qmin[i] = c->ha.exps[c->ha.pstart[i]];
     for (int k = 1; k < c->ha.nprim[i]; ++k) qmin[i] = std::min(qmin[i], c->ha.exps[c->ha.pstart[i] + k]);
   }
-  build_task_groups(c->pairs_h, c->hp.l, c->hp.nprim, c->ha.l, c->ha.nprim, pmax, qmin, tasks, se, sg);
   task_flops(c->pairs_h, c->hp.l, c->hp.nprim, c->hp.atom, c->ha.l, c->ha.nprim, c->ha.atom, c->nf_h, pmax, qmin,
              &c->flops_eri3, &c->flops_grad3);
+  build_task_groups(c->pairs_h, c->hp.l, c->hp.nprim, c->ha.l, c->ha.nprim, pmax, qmin, tasks, se, sg);
   size_t off = 0;
   for (int g = 0; g < kTaskGroups; ++g) {
     c->groups[g].tasks = c->d_tasks + off;
@@ -710,7 +742,7 @@ static void free_all(rihf_ctx* c) {
                   c->d_ao_atom, c->d_ao_l, c->hist_D[0], c->hist_D[1], c->hist_D[2], c->hist_S, c->hist_xyz[0],
                   c->hist_xyz[1], c->Shalf, c->Smhalf, c->DL, c->Dpred, c->mlX, c->mly, c->mlt, c->mlDx, c->ml_sums, c->rep_X, c->rep_t, c->net.master, c->net.wbf, c->net.grad,
                   c->net.m, c->net.v, c->net.loss,
-                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_flag, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_schwarz,
+                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_flag, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_chunks, c->d_ket, c->d_schwarz,
                   c->S, c->H, c->Tk, c->V, c->A, c->L, c->Linv, c->Bp, c->Yp, c->Bu, c->Dp, c->Jp, c->Xo, c->Sw, c->Sv,
                   c->C, c->eps, c->Ct, c->D, c->J, c->K, c->F, c->Fx, c->T1, c->T2, c->Err, c->Fp, c->Cp, c->Hb,
                   c->dvec, c->Fring, c->Ering, c->Bdiis, c->coef, c->scal, c->Cprev,
@@ -720,6 +752,26 @@ static void free_all(rihf_ctx* c) {
     if (p) cudaFree(p);
   for (OzBuf* b : {&c->Bz, &c->Cz, &c->Hz, &c->Ctz, &c->Gz, &c->Xz, &c->trsm_sc.L, &c->trsm_sc.X, &c->tcA, &c->tcB})
     oz_buf_free(*b);
+}
+
+// The geometry's lane-task descriptor, integrals into out or derivatives with Y into out.
+static LaneTasks lane_tasks(const rihf_ctx* c, double* out, const double* Y) {
+  LaneTasks t = c->lane;
+  t.geom.prim = c->prim();
+  t.geom.aux = c->aux();
+  t.geom.pairs = c->d_pairs;
+  t.geom.ptab = c->ptab();
+  t.geom.tasks = c->d_tasks;
+  t.geom.ket = c->d_ket;
+  t.geom.out = out;
+  t.geom.Y = Y;
+  return t;
+}
+
+// (mu nu|P) of every listed pair into the packed tensor T (the basis decides the kernels).
+static void eri3_all(rihf_ctx* c, double* T) {
+  if (c->opt.pure) launch_lane_eri3(c->ic(), c->sms, lane_tasks(c, T, nullptr));
+  else launch_eri3(c->ic(), c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, T);
 }
 
 // Geometry-dependent part of setup: shell centres, one-electron, metric,
@@ -806,7 +858,7 @@ static void compute_geometry(rihf_ctx* c, bool defer_eri3 = false) {
   }
   { TraceScope t(c->tracer, s, "eri3_kernel (mu nu|P)", c->flops_eri3, 0);
     launch_pair_prims(ic, P, c->d_pairs, c->npairs, c->d_pp_off, c->d_pp);
-    launch_eri3(ic, P, X, c->d_pairs, c->ptab(), c->groups, kTaskGroups, c->Bp); }
+    eri3_all(c, c->Bp); }
   compute_geometry_rest(c);
 }
 
@@ -1062,6 +1114,12 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
     c->d_tasks = dalloc<int2>(c->pairs_h.size() * (size_t)c->ha.nshell);
     c->d_pp_off = dalloc<int>(c->pairs_h.size() + 1);
     c->d_pp = dalloc<PairPrim>(std::max(1, pair_prim_offsets(c->pairs_h, c->hp.nprim).back()));
+    {
+      const std::vector<KetTable> ket = build_ket_tables(c->tr_h, c->nf_h);
+      c->d_ket = dalloc<KetTable>(ket.size());
+      upload(c->d_ket, ket, s);
+      RIHF_CUDA(cudaStreamSynchronize(s));
+    }
     refresh_tasks(c);
     {
       int maxsm = 0;
@@ -2534,7 +2592,8 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
     launch_grad_one_electron(ic, c->prim(), c->max_lp, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl); }
   if (!defer_eri3) {
     TraceScope t(c->tracer, s, "grad_eri3_kernel (fused d(mu nu|P) . Y)", c->flops_grad3, 0);
-    launch_grad_eri3(ic, c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, c->Yp, g_three);
+    if (c->opt.pure) launch_lane_grad(ic, c->sms, lane_tasks(c, g_three, c->Yp));
+    else launch_grad_eri3(ic, c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, c->Yp, g_three);
   }
   { TraceScope t(c->tracer, s, "grad_eri2_kernel (fused d(P|Q) . Z)", (double)NA * NA * 8, 1);
     launch_grad_eri2(ic, c->aux(), c->max_la, c->Zm, g_two); }
@@ -2633,7 +2692,7 @@ int rihf_get_matrix(rihf_ctx* c, int which, double* out) {
         double* tmp = dalloc<double>(pk.size());
         try {
           RIHF_CUDA(cudaMemsetAsync(tmp, 0, sizeof(double) * pk.size(), c->stream));
-          launch_eri3(c->ic(), c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, tmp);
+          eri3_all(c, tmp);
           RIHF_CUDA(cudaMemcpyAsync(pk.data(), tmp, sizeof(double) * pk.size(), cudaMemcpyDeviceToHost, c->stream));
           RIHF_CUDA(cudaStreamSynchronize(c->stream));
         } catch (...) {
@@ -2828,17 +2887,21 @@ int rihf_batch_step(int nmol, rihf_ctx* const* ctx, const double* const* xyz, in
   // stream then waits for
   cudaStream_t bs = nullptr;
   BatchTables tab;
+  LaneBatchTables ltab;
   int* bcount = nullptr;
   std::vector<cudaEvent_t> evs;
   auto release = [&]() {
     if (tab.geoms) cudaFree(tab.geoms);
     if (tab.off) cudaFree(tab.off);
+    if (ltab.geoms) cudaFree(ltab.geoms);
+    if (ltab.off) cudaFree(ltab.off);
     if (bcount) cudaFree(bcount);
     for (auto e : evs) cudaEventDestroy(e);
     if (bs) cudaStreamDestroy(bs);
   };
   auto batched_launch = [&](bool grad) -> bool {
-    std::vector<BatchGeom> batch;
+    std::vector<BatchGeom> batch;     // Cartesian members have tasks here,
+    std::vector<LaneTasks> lanes;     // spherical ones here
     std::vector<int> members;
     for (int i = 0; i < nmol; ++i) {
       if (rc[i] != RIHF_OK) continue;
@@ -2852,6 +2915,7 @@ int rihf_batch_step(int nmol, rihf_ctx* const* ctx, const double* const* xyz, in
       b.g.Y = grad ? c->Yp : nullptr;
       b.groups = c->groups;
       batch.push_back(b);
+      lanes.push_back(lane_tasks(c, b.g.out, b.g.Y));
       members.push_back(i);
     }
     if (batch.empty()) return true;
@@ -2866,10 +2930,12 @@ int rihf_batch_step(int nmol, rihf_ctx* const* ctx, const double* const* xyz, in
       ic.launches = nullptr;
       if (grad) launch_grad_eri3_batch(ic, batch, kTaskGroups, tab);
       else launch_eri3_batch(ic, batch, kTaskGroups, tab);
+      if (grad) launch_lane_grad_batch(ic, ctx[members[0]]->sms, lanes, ltab);
+      else launch_lane_eri3_batch(ic, ctx[members[0]]->sms, lanes, ltab);
       RIHF_CUDA(cudaEventRecord(evs[nmol], bs));
       for (int i : members) {
         RIHF_CUDA(cudaStreamWaitEvent(ctx[i]->stream, evs[nmol], 0));
-        ctx[i]->launches += kTaskGroups;
+        ctx[i]->launches += ctx[i]->opt.pure ? kLaneGroups : kTaskGroups;
       }
     } catch (const RihfError& e) {
       g_last_error = std::string("batched launch: ") + e.what();
@@ -2886,7 +2952,10 @@ int rihf_batch_step(int nmol, rihf_ctx* const* ctx, const double* const* xyz, in
     tab.cap = nmol;
     ok = ok && cudaMalloc(&tab.geoms, sizeof(GeomTasks) * (size_t)kTaskGroups * nmol) == cudaSuccess;
     ok = ok && cudaMalloc(&tab.off, sizeof(long long) * (size_t)kTaskGroups * (nmol + 1)) == cudaSuccess;
-    ok = ok && cudaMalloc(&bcount, sizeof(int)) == cudaSuccess;
+    ltab.cap = nmol;
+    ok = ok && cudaMalloc(&ltab.geoms, sizeof(LaneGeom) * (size_t)kLaneGroups * nmol) == cudaSuccess;
+    ok = ok && cudaMalloc(&ltab.off, sizeof(long long) * (size_t)kLaneGroups * (nmol + 1)) == cudaSuccess;
+    ok = ok && cudaMalloc(&bcount, kLaneGroups * sizeof(int)) == cudaSuccess;
     evs.resize(nmol + 1);
     for (auto& e : evs) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
