@@ -805,7 +805,7 @@ static void compute_geometry(rihf_ctx* c, bool defer_eri3 = false) {
       c->vnn += c->Z[a] * c->Z[b] / std::sqrt(r2);
     }
   RIHF_CUDA(cudaMemcpyAsync(c->scal + 5, &c->vnn, sizeof(double), cudaMemcpyHostToDevice, s));
-  RIHF_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
+  RIHF_CUDA(cudaMemsetAsync(c->d_flag, 0, 2 * sizeof(int), s));
   cudaEventRecord(c->ev[0], s);
   DevShells P = c->prim(), X = c->aux();
   { TraceScope t(c->tracer, s, "one_electron_kernel (S,T,V)", 3.0 * N * N * 8, 1);
@@ -915,7 +915,10 @@ static void compute_geometry_rest(rihf_ctx* c) {
     eigh(la, c->S, N, c->Sw, c->Sv, c->eigws, 4, nullptr);
     sw.resize(N);
     RIHF_CUDA(cudaMemcpyAsync(sw.data(), c->Sw, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
+    int late = 0;
+    RIHF_CUDA(cudaMemcpyAsync(&late, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaStreamSynchronize(s));
+    if (late) throw RihfError(RIHF_ERR_TIMEOUT, "overlap eigenvalues: a bounded device wait ran out");
     while (k0 < N && sw[k0] <= c->opt.lindep_tau) ++k0;
     if (k0 == N) throw RihfError(RIHF_ERR_NOT_POSITIVE_DEFINITE, "overlap matrix has no eigenvalue above lindep_tau");
   }
@@ -3147,16 +3150,18 @@ int rihf_eigh(int n, const double* A, double* W, double* V, int device) {
   size_t work_elems = std::max<size_t>((size_t)1 << 22, 8 * n2);
   try {
     dA = dalloc<double>(n2); dW = dalloc<double>(n); dV = dalloc<double>(n2);
-    ws = dalloc<double>(eig_workspace(n)); work = dalloc<double>(work_elems); flag = dalloc<int>(1);
+    ws = dalloc<double>(eig_workspace(n)); work = dalloc<double>(work_elems); flag = dalloc<int>(4);
+    RIHF_CUDA(cudaMemsetAsync(flag, 0, 4 * sizeof(int), s));
     RIHF_CUDA(cudaMemcpyAsync(dA, A, n2 * 8, cudaMemcpyHostToDevice, s));
     LaCtx la;
     la.stream = s; la.work = work; la.work_elems = work_elems; la.sms = sms; la.flag = flag;
-    // above order 1024 the block Jacobi's FP32 start carries the rounding of
-    // more rounds: two more refinement steps
-    eigh(la, dA, n, dW, dV, ws, n > 1024 ? 6 : 4, nullptr);
+    eigh(la, dA, n, dW, dV, ws, 4, nullptr);
+    int hflag[4];
+    RIHF_CUDA(cudaMemcpyAsync(hflag, flag, sizeof(hflag), cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaMemcpyAsync(W, dW, n * 8, cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaMemcpyAsync(V, dV, n2 * 8, cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaStreamSynchronize(s));
+    if (hflag[1]) throw RihfError(RIHF_ERR_TIMEOUT, "eigensolver: a grid barrier ran out of time");
   } catch (...) {
     cudaFree(dA); cudaFree(dW); cudaFree(dV); cudaFree(ws); cudaFree(work); cudaFree(flag);
     cudaStreamDestroy(s);
