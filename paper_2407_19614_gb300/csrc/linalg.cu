@@ -1129,7 +1129,7 @@ __global__ void oa_norms_kernel(const double* R, const double* S, const double* 
 
 __global__ void oa_e_kernel(const double* R, const double* S, const double* lam, const double* part, int nparts,
                             int n, double* E) {
-  __shared__ double sh_delta;
+  __shared__ double sh_delta, sh_min;
   if (threadIdx.x < 32) {   // fold the partial sums (fixed order: deterministic)
     double s0 = 0, s1 = 0, s2 = 0;
     for (int b = threadIdx.x; b < nparts; b += 32) {
@@ -1142,23 +1142,29 @@ __global__ void oa_e_kernel(const double* R, const double* S, const double* lam,
       s1 += __shfl_xor_sync(0xffffffffu, s1, o);
       s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     }
-    if (threadIdx.x == 0) sh_delta = 2.0 * (sqrt(s0) + sqrt(s2) * sqrt(s1));
+    if (threadIdx.x == 0) {
+      sh_delta = 2.0 * (sqrt(s0) + sqrt(s2) * sqrt(s1));
+      sh_min = 1e-14 * sqrt(s2);
+    }
   }
   __syncthreads();
-  const double delta = sh_delta;
+  const double delta = sh_delta, dmin = sh_min;
   // A pair is rotated when its gap exceeds the global cluster threshold (as in
   // the method), or when its own first-order correction is small, |E_ij| < 1/8.
   // The threshold bounds the spectral norms of the residuals by their
   // Frobenius norms, which for large n exceed them by up to sqrt(n): pairs far
   // apart relative to their own coupling would otherwise count as clustered and
   // never rotate (at n = 1856 the refinement then stalls near FP32 accuracy).
+  // A gap that is rounding of the norm (equal eigenvalues) says nothing: the
+  // quotient of two rounding errors would rotate by up to 1/8 at random and leave
+  // the vectors orthonormal to 1e-10 only.
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < (long long)n * n;
        idx += (long long)gridDim.x * blockDim.x) {
     int i = (int)(idx / n), j = (int)(idx % n);
     double r = R[idx];
     const double num = S[idx] + lam[j] * r, dl = lam[j] - lam[i];
     double e;
-    if (i != j && (fabs(dl) > delta || fabs(dl) > 8.0 * fabs(num))) e = num / dl;
+    if (i != j && fabs(dl) > dmin && (fabs(dl) > delta || fabs(dl) > 8.0 * fabs(num))) e = num / dl;
     else e = 0.5 * r;
     E[idx] = e;
   }
@@ -1183,16 +1189,21 @@ static int elem_blocks(const LaCtx& la, long long n) {
 }
 
 // Ascending reorder of FP64 eigenpairs: Vout[:, rank(i)] = V[:, i], Wout[rank(i)] = lam[i].
+// Ranks by integer comparison of order-preserving keys: n^2 FP64 comparisons hold the
+// FP64 pipe (257 us at n = 580 with them, every block ranking all values).
 __global__ void eig_sort64_kernel(const double* __restrict__ V, const double* __restrict__ lam, int n, double* Vout,
                                   double* Wout) {
+  __shared__ unsigned long long key[4096];
   __shared__ int rank[4096];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    double wi = lam[i];
+    const unsigned long long b = (unsigned long long)__double_as_longlong(lam[i] + 0.0);   // -0 as +0
+    key[i] = b >> 63 ? ~b : b | 1ull << 63;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    const unsigned long long wi = key[i];
     int r = 0;
-    for (int j = 0; j < n; ++j) {
-      double wj = lam[j];
-      if (wj < wi || (wj == wi && j < i)) ++r;
-    }
+    for (int j = 0; j < n; ++j) r += key[j] < wi || (key[j] == wi && j < i);
     rank[i] = r;
   }
   __syncthreads();

@@ -131,9 +131,9 @@ constexpr size_t eig_workspace_base(int n) {
          6 * (size_t)n * n + 2 * (size_t)n + 8;
 }
 // Doubles of tridiag_eigh: the reflectors, the tridiagonal's eigenvectors, four
-// factor arrays (one of them first holds the working rows), d, e, tau, the
+// factor arrays (one of them first holds the working rows), d, e, e^2, tau, the
 // published vectors, norms, block ranges and the barrier counter.
-constexpr size_t tridiag_workspace(int n) { return 6 * (size_t)n * n + 9 * (size_t)n + 16; }
+constexpr size_t tridiag_workspace(int n) { return 6 * (size_t)n * n + 10 * (size_t)n + 16; }
 constexpr size_t eig_workspace(int n) { return eig_workspace_base(n) + (n > kJacobiMax ? tridiag_workspace(n) : 0); }
 // skip_jacobi: start the refinement from Vguess directly (late SCF iterations).
 // max_sweeps caps the FP32 Jacobi sweeps and ns_steps the Newton-Schulz
