@@ -1,6 +1,9 @@
 // Dense linear algebra kernels of librihf.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "../../include/rihf.h"
 #include "eigh_tridiag.cuh"
@@ -35,87 +38,139 @@ static inline void count(const LaCtx& la, int n = 1) {
 
 // ------------------------------------------------------------ GEMM (FP64)
 
-constexpr int GT = 32;   // output tile
-constexpr int GK = 16;   // K step
+// C tiles of 16 x 16 by 128-thread CTAs, two elements a thread.  FP64 bounds every
+// product here (two FMAs per clock and SM), so what counts is that no tile is
+// mostly padding and that the tiles fill the SMs evenly: 16 is the largest tile
+// that gives a 192 x 192 result one CTA per SM (144) without splitting K, and wastes
+// least at the 40 columns of H = B C~ (48 computed; 64 with a 32-wide tile).  The
+// operands come through a ring of three K chunks filled by cp.async two chunks
+// ahead.  Measured, 192 x 192 x 192: 18 us, 14 us for a symmetric result, against
+// 17 us plus a 5 us reduction of split sums with 32 x 32 tiles; H and K of an FP64
+// Fock build at N = 192, Naux = 848 (40 occupied): 3.6 ms against 5.7.
+constexpr int GT = 16;        // output tile
+constexpr int GK = 32;        // K chunk, at most
+constexpr int GS = 3;         // chunks in flight
+constexpr int GThreads = 128;
+constexpr int kGemmCluster = 8;   // most K slices summed through a thread-block cluster
 
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) dgemm_kernel(GemmArgs g, int nsplit, int kper, int bper,
-                                                    double* __restrict__ work) {
-  __shared__ double As[GK][GT + 1];
-  __shared__ double Bs[GK][GT + 1];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int n0 = blockIdx.x * GT, m0 = blockIdx.y * GT;
-  const int z = blockIdx.z;
-  if (g.symcols > 0) {
-    int j0 = n0, j1 = min(n0 + GT, g.N) - 1;
-    bool spans = (j0 / g.symcols) != (j1 / g.symcols);
-    if (!spans && (j0 % g.symcols) > (j0 / g.symcols)) return;
+// Eight-byte asynchronous copy; zero when the element does not exist.
+__device__ __forceinline__ void gemm_cp8(double* dst, const double* src, bool valid) {
+  const unsigned at = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = valid ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(at), "l"(src), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void gemm_store(const GemmArgs& g, double* C, int m, int n, double v) {
+  if (m >= g.M || n >= g.N) return;
+  double* c = C + (long long)m * g.ldc + n;
+  *c = g.beta == 0.0 ? g.alpha * v : g.alpha * v + g.beta * *c;
+}
+
+// Tile t of the result: all tiles row by row, or (lower_only) those on and below
+// the diagonal.
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int t, int tn, int& tm, int& tc) {
+  if (!g.lower_only) {
+    tm = t / tn;
+    tc = t - tm * tn;
+    return;
   }
-  if (g.lower_only && n0 > m0) return;
-  int b_lo, b_hi, k_lo, k_hi, slot_b, slot_s;
+  tm = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+  while (tm * (tm + 1) / 2 > t) --tm;
+  while ((tm + 1) * (tm + 2) / 2 <= t) ++tm;
+  tc = t - tm * (tm + 1) / 2;
+}
+
+// grid.x: tiles x batches; grid.y: slices of the sum (K, or the batches when they
+// are reduced).  Slices are summed in order: in a cluster over the slices through
+// distributed shared memory (each CTA a part of the tile), or by
+// splitk_reduce_kernel from `work` when there are more than a cluster holds.
+// FULL: chunks of GK (K a multiple of it), whose index arithmetic needs no division.
+template <bool TA, bool TB, bool FULL>
+__global__ void __launch_bounds__(GThreads) dgemm_kernel(GemmArgs g, int tiles, int tn, int nslice, int kper, int bper,
+                                                         int chunk_, int cluster, double* __restrict__ work) {
+  const int chunk = FULL ? GK : chunk_;
+  __shared__ double As[GS][GK][GT + 1], Bs[GS][GK][GT + 1];
+  __shared__ double part[GT * GT];
+  const int tid = threadIdx.x;
+  const int batch = blockIdx.x / tiles, slice = blockIdx.y;
+  int tm, tc;
+  gemm_tile(g, blockIdx.x - batch * tiles, tn, tm, tc);
+  const int m0 = tm * GT, n0 = tc * GT;
+  int b0 = batch, b1 = batch + 1, k0 = 0, k1 = g.K;
   if (g.reduce_batch) {
-    slot_s = z;
-    slot_b = 0;
-    b_lo = z * bper;
-    b_hi = min(g.batch, b_lo + bper);
-    k_lo = 0;
-    k_hi = g.K;
+    b0 = slice * bper;
+    b1 = min(g.batch, b0 + bper);
   } else {
-    slot_b = z / nsplit;
-    slot_s = z % nsplit;
-    b_lo = slot_b;
-    b_hi = slot_b + 1;
-    k_lo = slot_s * kper;
-    k_hi = min(g.K, k_lo + kper);
+    k0 = slice * kper;
+    k1 = min(g.K, k0 + kper);
   }
-  if (g.lowerA) k_hi = min(k_hi, m0 + GT);
-  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  for (int b = b_lo; b < b_hi; ++b) {
-    const double* A = g.A + (long long)b * g.sA;
-    const double* B = g.B + (long long)b * g.sB;
-    for (int k0 = k_lo; k0 < k_hi; k0 += GK) {
-      for (int r = 0; r < 2; ++r) {
-        int idx = tid + r * 256;
-        int mm, kk;
-        if (TA) { mm = idx % GT; kk = idx / GT; } else { kk = idx % GK; mm = idx / GK; }
-        int m = m0 + mm, k = k0 + kk;
-        double v = 0.0;
-        if (m < g.M && k < k_hi) v = TA ? A[(long long)k * g.lda + m] : A[(long long)m * g.lda + k];
-        As[kk][mm] = v;
-        int nn, kb;
-        if (TB) { kb = idx % GK; nn = idx / GK; } else { nn = idx % GT; kb = idx / GT; }
-        int n = n0 + nn, kq = k0 + kb;
-        double w = 0.0;
-        if (n < g.N && kq < k_hi) w = TB ? B[(long long)n * g.ldb + kq] : B[(long long)kq * g.ldb + n];
-        Bs[kb][nn] = w;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < GK; ++kk) {
-        double a0 = As[kk][ty * 2], a1 = As[kk][ty * 2 + 1];
-        double b0 = Bs[kk][tx * 2], b1 = Bs[kk][tx * 2 + 1];
-        acc[0][0] = fma(a0, b0, acc[0][0]);
-        acc[0][1] = fma(a0, b1, acc[0][1]);
-        acc[1][0] = fma(a1, b0, acc[1][0]);
-        acc[1][1] = fma(a1, b1, acc[1][1]);
-      }
-      __syncthreads();
-    }
-  }
-  const bool direct = g.reduce_batch ? (gridDim.z == 1) : (nsplit == 1);
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) {
-      int m = m0 + ty * 2 + i, n = n0 + tx * 2 + j;
-      if (m >= g.M || n >= g.N) continue;
-      if (direct) {
-        double* C = g.C + (g.reduce_batch ? 0 : (long long)slot_b * g.sC);
-        double* c = C + (long long)m * g.ldc + n;
-        *c = g.beta == 0.0 ? g.alpha * acc[i][j] : g.alpha * acc[i][j] + g.beta * *c;
-      } else {
-        long long slot = (long long)slot_b * (g.reduce_batch ? gridDim.z : nsplit) + slot_s;
-        work[slot * g.M * g.N + (long long)m * g.N + n] = acc[i][j];
+  const int per = k1 > k0 ? (k1 - k0 + chunk - 1) / chunk : 0;   // chunks of one batch
+  const int total = b1 > b0 ? (b1 - b0) * per : 0;
+  auto fetch = [&](int c) {
+    if (c < total) {
+      const int b = b0 + c / per, kc = k0 + (c % per) * chunk;
+      const double* A = g.A + (long long)b * g.sA;
+      const double* B = g.B + (long long)b * g.sB;
+      const int st = c % GS;
+      for (int idx = tid; idx < GT * chunk; idx += GThreads) {
+        int mm, ka, nn, kb;
+        if (TA) { mm = idx % GT; ka = idx / GT; } else { ka = idx % chunk; mm = idx / chunk; }
+        if (TB) { kb = idx % chunk; nn = idx / chunk; } else { nn = idx % GT; kb = idx / GT; }
+        const int m = m0 + mm, n = n0 + nn, x = kc + ka, y = kc + kb;
+        const bool va = m < g.M && x < k1, vb = n < g.N && y < k1;
+        gemm_cp8(&As[st][ka][mm], va ? (TA ? A + (long long)x * g.lda + m : A + (long long)m * g.lda + x) : A, va);
+        gemm_cp8(&Bs[st][kb][nn], vb ? (TB ? B + (long long)n * g.ldb + y : B + (long long)y * g.ldb + n) : B, vb);
       }
     }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  const int tx = tid % 8, ty = tid / 8;   // row ty, columns 2 tx, 2 tx + 1
+  double acc0 = 0.0, acc1 = 0.0;
+  for (int c = 0; c < GS - 1; ++c) fetch(c);
+  for (int c = 0; c < total; ++c) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(GS - 2) : "memory");
+    __syncthreads();   // chunk c has arrived; the stage of chunk c - 1 is free
+    fetch(c + GS - 1);
+    const int st = c % GS, kc = k0 + (c % per) * chunk, kv = min(chunk, k1 - kc);
+#pragma unroll 8
+    for (int k = 0; k < kv; ++k) {
+      const double a = As[st][k][ty];
+      acc0 = fma(a, Bs[st][k][2 * tx], acc0);
+      acc1 = fma(a, Bs[st][k][2 * tx + 1], acc1);
+    }
+  }
+  if (nslice > 1 && !cluster) {
+    const long long slot = (long long)batch * nslice + slice;
+    const int m = m0 + ty, n = n0 + 2 * tx;
+    double* w = work + slot * g.M * g.N + (long long)m * g.N + n;
+    if (m < g.M && n < g.N) w[0] = acc0;
+    if (m < g.M && n + 1 < g.N) w[1] = acc1;
+    return;
+  }
+  double* C = g.C + (g.reduce_batch ? 0 : (long long)batch * g.sC);
+  if (nslice > 1) {
+    namespace cg = cooperative_groups;
+    auto cl = cg::this_cluster();
+    part[ty * GT + 2 * tx] = acc0;
+    part[ty * GT + 2 * tx + 1] = acc1;
+    cl.sync();
+    for (int e = slice * GThreads + tid; e < GT * GT; e += nslice * GThreads) {
+      double s = 0.0;
+      for (int q = 0; q < nslice; ++q) s += *cl.map_shared_rank(part + e, q);
+      const int m = m0 + e / GT, n = n0 + e % GT;
+      gemm_store(g, C, m, n, s);
+      if (g.mirror && n0 < m0) gemm_store(g, C, n, m, s);
+    }
+    cl.sync();   // no CTA leaves while its partial tile is read
+    return;
+  }
+  const int m = m0 + ty, n = n0 + 2 * tx;
+  gemm_store(g, C, m, n, acc0);
+  gemm_store(g, C, m, n + 1, acc1);
+  if (g.mirror && n0 < m0) {
+    gemm_store(g, C, n, m, acc0);
+    gemm_store(g, C, n + 1, m, acc1);
+  }
 }
 
 __global__ void splitk_reduce_kernel(GemmArgs g, int nsplit, const double* __restrict__ work) {
@@ -125,17 +180,12 @@ __global__ void splitk_reduce_kernel(GemmArgs g, int nsplit, const double* __res
     long long mn = idx % ((long long)g.M * g.N);
     int b = (int)(idx / ((long long)g.M * g.N));
     int m = (int)(mn / g.N), n = (int)(mn % g.N);
-    if (g.symcols > 0) {
-      // tiles skipped in the product were never written; mirror does the rest
-      int j0 = (n / GT) * GT, j1 = min(j0 + GT, g.N) - 1;
-      bool spans = (j0 / g.symcols) != (j1 / g.symcols);
-      if (!spans && (j0 % g.symcols) > (j0 / g.symcols)) continue;
-    }
     if (g.lower_only && (n / GT) > (m / GT)) continue;
     double s = 0.0;
     for (int q = 0; q < nsplit; ++q) s += work[((long long)b * nsplit + q) * g.M * g.N + mn];
-    double* c = g.C + (g.reduce_batch ? 0 : (long long)b * g.sC) + (long long)m * g.ldc + n;
-    *c = g.beta == 0.0 ? g.alpha * s : g.alpha * s + g.beta * *c;
+    double* C = g.C + (g.reduce_batch ? 0 : (long long)b * g.sC);
+    gemm_store(g, C, m, n, s);
+    if (g.mirror && (n / GT) < (m / GT)) gemm_store(g, C, n, m, s);
   }
 }
 
@@ -143,7 +193,7 @@ __global__ void splitk_reduce_kernel(GemmArgs g, int nsplit, const double* __res
 // op(B)^T as rows N, K, both sliced into 7 digits; C stored (beta 0) or
 // accumulated (beta 1).  Returns false when the product does not qualify.
 static bool dgemm_tc(const LaCtx& la, const GemmArgs& g) {
-  if (!la.tcA || !la.tcB || g.batch != 1 || g.reduce_batch || g.lowerA || g.symcols != 0 ||
+  if (!la.tcA || !la.tcB || g.batch != 1 || g.reduce_batch ||
       !(g.beta == 0.0 || g.beta == 1.0) || g.K <= 0)
     return false;
   if ((double)g.M * g.N * g.K < la.tc_min_work) return false;
@@ -166,200 +216,81 @@ static bool dgemm_tc(const LaCtx& la, const GemmArgs& g) {
 
 void dgemm(const LaCtx& la, const GemmArgs& g) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
-  if (dgemm_tc(la, g)) return;
-  int tm = ceil_div(g.M, GT), tn = ceil_div(g.N, GT);
-  if (tm > 65535) {
-    // row tiles run on grid.y (at most 65535): tall products (rows (P, mu) of
-    // Naux N) go in row slabs
-    if (g.batch != 1 || g.reduce_batch || g.lowerA || g.lower_only || g.symcols)
-      throw RihfError(RIHF_ERR_INVALID_ARG, "dgemm: too many row tiles for this product shape");
-    const int slab = 65535 * GT;
-    for (int r0 = 0; r0 < g.M; r0 += slab) {
-      GemmArgs h = g;
-      h.M = std::min(slab, g.M - r0);
-      h.A = g.A + (size_t)r0 * (g.transA ? 1 : g.lda);
-      h.C = g.C + (size_t)r0 * g.ldc;
-      dgemm(la, h);
-    }
+  if (dgemm_tc(la, g)) {
+    if (g.mirror) symmetrize_lower(la, g.C, g.N, 1);
     return;
   }
-  long long tiles = (long long)tm * tn * (g.reduce_batch ? 1 : g.batch);
-  int nsplit = 1, kper = g.K, bper = g.batch;
-  const long long target = 4LL * la.sms;
+  const int tm = ceil_div(g.M, GT), tn = ceil_div(g.N, GT);
+  const int nb = g.reduce_batch ? 1 : g.batch;
+  if ((long long)tm * tn > 0x7fffffffLL / nb)
+    throw RihfError(RIHF_ERR_INVALID_ARG, "dgemm: too many tiles for this product shape");
+  const int tiles = g.lower_only ? tm * (tm + 1) / 2 : tm * tn;
+  // the chunk divides K when K is short (reduced batches of K = nocc: no padded steps)
+  const int chunk = std::max(1, ceil_div(g.K, ceil_div(std::max(1, g.K), GK)));
+  // Slices: the least time of the fullest SM, in FP64 steps of one tile: a CTA alone
+  // on its SM takes 1.75 times its FP64 time (one warp per sub-partition: 226 clocks
+  // a step instead of 128, measured at 192 x 192 x 192), so two half slices beat one
+  // whole; and a slice costs some steps beside its own (filling the ring, the sum).
+  // Up to kGemmCluster slices are summed in a cluster; more go through la.work, which
+  // has to hold them, and only where a long reduction leaves each slice long.
+  const long long ctas = (long long)tiles * nb;
+  const long long len = g.reduce_batch ? (long long)g.batch * g.K : g.K;
+  const long long most_len = g.reduce_batch ? g.batch : std::max(1, g.K / 8);   // at least 8 of K a slice
+  int nslice = 1;
+  double best = 1e300;
+  for (int s = 1; s <= 64 && s <= most_len; ++s) {
+    if (s > kGemmCluster &&
+        ((size_t)s * g.M * g.N * nb > la.work_elems || len / s < 512)) break;
+    const double steps = (double)ceil_div(len, s) + (s > 1 ? 16.0 : 8.0) + (s > kGemmCluster ? 40.0 : 0.0);
+    const double cost = std::max((double)((ctas * s + la.sms - 1) / la.sms), 1.75) * steps;
+    if (cost < 0.98 * best) {
+      best = cost;
+      nslice = s;
+    }
+  }
+  int kper = g.K, bper = g.batch;
   if (g.reduce_batch) {
-    nsplit = (int)std::min<long long>(g.batch, std::max<long long>(1, (target + tiles - 1) / tiles));
-    while (nsplit > 1 && (size_t)nsplit * g.M * g.N > la.work_elems) nsplit /= 2;
-    bper = ceil_div(g.batch, nsplit);
-    nsplit = ceil_div(g.batch, bper);
-  } else if (tiles < target && g.K > 2 * GK) {
-    nsplit = (int)std::min<long long>((target + tiles - 1) / tiles, g.K / GK);
-    while (nsplit > 1 && (size_t)nsplit * g.M * g.N * g.batch > la.work_elems) nsplit /= 2;
-    kper = ceil_div(ceil_div(g.K, nsplit), GK) * GK;
-    nsplit = ceil_div(g.K, kper);
+    bper = ceil_div(g.batch, nslice);
+    nslice = ceil_div(g.batch, bper);
+  } else if (nslice > 1) {
+    kper = ceil_div(g.K, nslice);
+    nslice = ceil_div(g.K, kper);
   }
-  if (g.lowerA && nsplit > 1 && !g.reduce_batch) {
-    // the triangular cut is per row tile; keep it simple and exact
-    nsplit = 1;
-    kper = g.K;
+  const int cluster = nslice > 1 && nslice <= kGemmCluster ? 1 : 0;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  cfg.gridDim = dim3((unsigned)ctas, (unsigned)nslice, 1);
+  cfg.blockDim = dim3(GThreads, 1, 1);
+  cfg.stream = la.stream;
+  if (cluster) {
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1;
+    attr.val.clusterDim.y = (unsigned)nslice;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
   }
-  dim3 grid(tn, tm, g.reduce_batch ? nsplit : g.batch * nsplit);
-  if (g.transA && g.transB)
-    dgemm_kernel<true, true><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, la.work);
-  else if (g.transA)
-    dgemm_kernel<true, false><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, la.work);
-  else if (g.transB)
-    dgemm_kernel<false, true><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, la.work);
-  else
-    dgemm_kernel<false, false><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, la.work);
-  RIHF_LAUNCH_CHECK();
+  auto run = [&](auto kernel) {
+    RIHF_CUDA(cudaLaunchKernelEx(&cfg, kernel, g, tiles, tn, nslice, kper, bper, chunk, cluster, la.work));
+  };
+  auto pick = [&](auto full) {
+    constexpr bool F = decltype(full)::value;
+    if (g.transA && g.transB) run(dgemm_kernel<true, true, F>);
+    else if (g.transA) run(dgemm_kernel<true, false, F>);
+    else if (g.transB) run(dgemm_kernel<false, true, F>);
+    else run(dgemm_kernel<false, false, F>);
+  };
+  if (chunk == GK) pick(std::true_type());
+  else pick(std::false_type());
   count(la);
-  if (nsplit > 1) {
-    long long total = (long long)g.M * g.N * (g.reduce_batch ? 1 : g.batch);
-    int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * la.sms);
-    splitk_reduce_kernel<<<blocks, 256, 0, la.stream>>>(g, nsplit, la.work);
+  if (nslice > 1 && !cluster) {
+    const long long total = (long long)g.M * g.N * nb;
+    const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * la.sms);
+    splitk_reduce_kernel<<<blocks, 256, 0, la.stream>>>(g, nslice, la.work);
     RIHF_LAUNCH_CHECK();
     count(la);
   }
 }
-
-// ------------------------------------------------------------ GEMM (FP32)
-
-constexpr int ST = 64;   // output tile
-constexpr int SK = 16;   // K step
-
-template <bool TA, bool TB>
-__global__ void __launch_bounds__(256) sgemm_kernel(SGemmArgs g, int nsplit, int kper, int bper, float* work) {
-  __shared__ float As[SK][ST + 4];
-  __shared__ float Bs[SK][ST + 4];
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int n0 = blockIdx.x * ST, m0 = blockIdx.y * ST;
-  const int z = blockIdx.z;
-  int b_lo, b_hi, k_lo, k_hi, slot_b, slot_s;
-  if (g.reduce_batch) {
-    slot_s = z; slot_b = 0; b_lo = z * bper; b_hi = min(g.batch, b_lo + bper); k_lo = 0; k_hi = g.K;
-  } else {
-    slot_b = z / nsplit; slot_s = z % nsplit; b_lo = slot_b; b_hi = slot_b + 1;
-    k_lo = slot_s * kper; k_hi = min(g.K, k_lo + kper);
-  }
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int b = b_lo; b < b_hi; ++b) {
-    const float* A = g.A + (long long)b * g.sA;
-    const float* B = g.B + (long long)b * g.sB;
-    for (int k0 = k_lo; k0 < k_hi; k0 += SK) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        int idx = tid + r * 256;   // 1024 = 64 x 16
-        int mm, kk;
-        if (TA) { mm = idx % ST; kk = idx / ST; } else { kk = idx % SK; mm = idx / SK; }
-        int m = m0 + mm, k = k0 + kk;
-        float v = 0.f;
-        if (m < g.M && k < k_hi) v = TA ? A[(long long)k * g.lda + m] : A[(long long)m * g.lda + k];
-        As[kk][mm] = v;
-        int nn, kb;
-        if (TB) { kb = idx % SK; nn = idx / SK; } else { nn = idx % ST; kb = idx / ST; }
-        int n = n0 + nn, kq = k0 + kb;
-        float w = 0.f;
-        if (n < g.N && kq < k_hi) w = TB ? B[(long long)n * g.ldb + kq] : B[(long long)kq * g.ldb + n];
-        Bs[kb][nn] = w;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < SK; ++kk) {
-        float a[4], bb[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) bb[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
-      }
-      __syncthreads();
-    }
-  }
-  const int nslots = g.reduce_batch ? (int)gridDim.z : nsplit;
-  const bool direct = nslots == 1;
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      int m = m0 + ty * 4 + i, n = n0 + tx * 4 + j;
-      if (m >= g.M || n >= g.N) continue;
-      if (direct && !g.Cd) {
-        float* c = g.C + (g.reduce_batch ? 0 : (long long)slot_b * g.sC) + (long long)m * g.ldc + n;
-        *c = (float)(g.beta == 0.0 ? g.alpha * acc[i][j] : g.alpha * acc[i][j] + g.beta * *c);
-      } else {
-        long long slot = (long long)slot_b * nslots + slot_s;
-        work[slot * g.M * g.N + (long long)m * g.N + n] = acc[i][j];
-      }
-    }
-}
-
-__global__ void sgemm_reduce_kernel(SGemmArgs g, int nslots, const float* __restrict__ work) {
-  long long total = (long long)g.M * g.N * (g.reduce_batch ? 1 : g.batch);
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    long long mn = idx % ((long long)g.M * g.N);
-    int b = (int)(idx / ((long long)g.M * g.N));
-    int m = (int)(mn / g.N), n = (int)(mn % g.N);
-    double s = 0.0;
-    for (int q = 0; q < nslots; ++q) s += (double)work[((long long)b * nslots + q) * g.M * g.N + mn];
-    long long off = (g.reduce_batch ? 0 : (long long)b * g.sC) + (long long)m * g.ldc + n;
-    if (g.Cd) g.Cd[off] = g.beta == 0.0 ? g.alpha * s : g.alpha * s + g.beta * g.Cd[off];
-    else g.C[off] = (float)(g.beta == 0.0 ? g.alpha * s : g.alpha * s + g.beta * g.C[off]);
-  }
-}
-
-void sgemm(const LaCtx& la, const SGemmArgs& g) {
-  if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
-  int tm = ceil_div(g.M, ST), tn = ceil_div(g.N, ST);
-  long long tiles = (long long)tm * tn * (g.reduce_batch ? 1 : g.batch);
-  int nsplit = 1, kper = g.K, bper = g.batch;
-  const long long target = 4LL * la.sms;
-  const size_t cap = la.work_elems * 2;   // the workspace holds twice as many floats
-  if (g.reduce_batch) {
-    nsplit = (int)std::min<long long>(g.batch, std::max<long long>(1, (target + tiles - 1) / tiles));
-    while (nsplit > 1 && (size_t)nsplit * g.M * g.N > cap) nsplit /= 2;
-    bper = ceil_div(g.batch, nsplit);
-    nsplit = ceil_div(g.batch, bper);
-  } else if (tiles < target && g.K > 4 * SK) {
-    nsplit = (int)std::min<long long>((target + tiles - 1) / tiles, g.K / (2 * SK));
-    while (nsplit > 1 && (size_t)nsplit * g.M * g.N * g.batch > cap) nsplit /= 2;
-    kper = ceil_div(ceil_div(g.K, nsplit), SK) * SK;
-    nsplit = ceil_div(g.K, kper);
-  }
-  float* work = reinterpret_cast<float*>(la.work);
-  dim3 grid(tn, tm, g.reduce_batch ? nsplit : g.batch * nsplit);
-  if (g.transA && g.transB) sgemm_kernel<true, true><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, work);
-  else if (g.transA) sgemm_kernel<true, false><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, work);
-  else if (g.transB) sgemm_kernel<false, true><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, work);
-  else sgemm_kernel<false, false><<<grid, 256, 0, la.stream>>>(g, nsplit, kper, bper, work);
-  RIHF_LAUNCH_CHECK();
-  count(la);
-  if (nsplit > 1 || g.Cd) {
-    long long total = (long long)g.M * g.N * (g.reduce_batch ? 1 : g.batch);
-    int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * la.sms);
-    sgemm_reduce_kernel<<<blocks, 256, 0, la.stream>>>(g, nsplit, work);
-    RIHF_LAUNCH_CHECK();
-    count(la);
-  }
-}
-
-__global__ void to_float_kernel(const double* __restrict__ in, long long n, float* __restrict__ out, double s) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = (float)(s * in[i]);
-}
-void to_float(const LaCtx& la, const double* in, long long n, float* out, double scale) {
-  int blocks = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 16LL * la.sms));
-  to_float_kernel<<<blocks, 256, 0, la.stream>>>(in, n, out, scale);
-  RIHF_LAUNCH_CHECK();
-  count(la);
-}
-
-// ------------------------------------------------------------ symmetrize
 
 __global__ void symmetrize_lower_kernel(double* X, int n) {
   __shared__ double t[32][33];
@@ -588,7 +519,6 @@ void trsm_lower(const LaCtx& la, const double* L, int n, double* X, long long nc
     u.N = (int)ncol; u.K = b;
     u.B = X + (size_t)k * ncol; u.ldb = (int)ncol;
     u.alpha = -1.0; u.beta = 1.0;
-    u.symcols = symcols;
     if (!trans) {
       // X[k+b:, :] -= L[k+b:, k:k+b] X_k
       u.M = n - k - b;
@@ -637,7 +567,7 @@ void trsm_lower_tc(const LaCtx& la, const double* L, int n, double* X, long long
         u.A = L + (size_t)(k2 + b) * n + k2; u.lda = n;
         u.B = X + (size_t)k2 * ncol; u.ldb = (int)ncol;
         u.C = X + (size_t)(k2 + b) * ncol; u.ldc = (int)ncol;
-        u.alpha = -1.0; u.beta = 1.0; u.symcols = symcols;
+        u.alpha = -1.0; u.beta = 1.0;
         dgemm(la, u);
       }
     }
@@ -682,7 +612,7 @@ void trsm_lower_t_tc(const LaCtx& la, const double* L, int n, double* X, long lo
           u.A = L + (size_t)k2 * n + k; u.lda = n; u.transA = true;
           u.B = X + (size_t)k2 * ncol; u.ldb = (int)ncol;
           u.C = X + (size_t)k * ncol; u.ldc = (int)ncol;
-          u.alpha = -1.0; u.beta = 1.0; u.symcols = symcols;
+          u.alpha = -1.0; u.beta = 1.0;
           dgemm(la, u);
         }
       }
@@ -1260,7 +1190,7 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
     dgemm(la, g1);
     GemmArgs g2;
     g2.M = n; g2.N = n; g2.K = n; g2.A = Vguess; g2.lda = n; g2.transA = true; g2.B = AX; g2.ldb = n;
-    g2.C = Ag; g2.ldc = n;
+    g2.C = Ag; g2.ldc = n; g2.lower_only = g2.mirror = true;
     dgemm(la, g2);
     Ain = Ag;
   }
@@ -1301,6 +1231,7 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
   for (int it = 0; it < refine; ++it) {
     GemmArgs gr;   // R = V^T V
     gr.M = n; gr.N = n; gr.K = n; gr.A = V; gr.lda = n; gr.transA = true; gr.B = V; gr.ldb = n; gr.C = R; gr.ldc = n;
+    gr.lower_only = gr.mirror = true;
     dgemm(la, gr);
     i_minus_kernel<<<elem_blocks(la, (long long)n * n), 256, 0, la.stream>>>(R, n);
     RIHF_LAUNCH_CHECK();
@@ -1309,6 +1240,7 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
     dgemm(la, ga);
     GemmArgs gs;   // S = V^T A V
     gs.M = n; gs.N = n; gs.K = n; gs.A = V; gs.lda = n; gs.transA = true; gs.B = AX; gs.ldb = n; gs.C = S; gs.ldc = n;
+    gs.lower_only = gs.mirror = true;
     dgemm(la, gs);
     oa_lambda_kernel<<<elem_blocks(la, n), 256, 0, la.stream>>>(R, S, n, lam);
     // partial norms in the XE slot (written only by the update GEMM below)
@@ -1332,7 +1264,7 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
     for (int it = 0; it < ns_steps; ++it) {
       GemmArgs gr;
       gr.M = n; gr.N = n; gr.K = n; gr.A = V; gr.lda = n; gr.transA = true; gr.B = V; gr.ldb = n; gr.C = R;
-      gr.ldc = n; gr.alpha = -0.5;
+      gr.ldc = n; gr.alpha = -0.5; gr.lower_only = gr.mirror = true;
       dgemm(la, gr);
       identity(la, E, n);
       axpby(la, n * n, 1.0, R, 1.5, E, R);

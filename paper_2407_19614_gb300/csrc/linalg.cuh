@@ -29,9 +29,8 @@ struct LaCtx {
 // op(A) is M x K: A[m*lda + k] (transA = false) or A[k*lda + m] (true);
 // op(B) is K x N: B[k*ldb + n] (transB = false) or B[n*ldb + k] (true).
 // reduce_batch: all batches accumulate into C[0] (C stride ignored).
-// lowerA: A is lower triangular (op(A)[m][k] = 0 for k > m), K-loop is cut.
-// symcols: > 0 skips column tiles whose every column j has (j % symcols) > (j / symcols)
-//          (strict upper triangle of an N x N slice flattened along columns).
+// lower_only: a symmetric result, computed on and below the diagonal (16 x 16 tiles);
+// mirror: and written to both triangles (with beta 0, or a symmetric C).
 struct GemmArgs {
   int M = 0, N = 0, K = 0;
   double alpha = 1.0, beta = 0.0;
@@ -48,36 +47,10 @@ struct GemmArgs {
   long long sC = 0;
   int batch = 1;
   bool reduce_batch = false;
-  bool lowerA = false;
-  int symcols = 0;
-  bool lower_only = false;   // symmetric result: compute tiles on/below the diagonal only
+  bool lower_only = false;
+  bool mirror = false;
 };
 void dgemm(const LaCtx& la, const GemmArgs& g);
-
-// FP32 operands, FP32 accumulation (CUDA cores, 64 x 64 tiles).  Same
-// conventions as GemmArgs; when Cd is set the result goes to the FP64 matrix Cd
-// (alpha * sum + beta * Cd, split partial sums added in FP64), else to C (FP32).
-struct SGemmArgs {
-  int M = 0, N = 0, K = 0;
-  double alpha = 1.0, beta = 0.0;
-  const float* A = nullptr;
-  int lda = 0;
-  long long sA = 0;
-  bool transA = false;
-  const float* B = nullptr;
-  int ldb = 0;
-  long long sB = 0;
-  bool transB = false;
-  float* C = nullptr;
-  double* Cd = nullptr;
-  int ldc = 0;
-  long long sC = 0;
-  int batch = 1;
-  bool reduce_batch = false;
-};
-void sgemm(const LaCtx& la, const SGemmArgs& g);
-// out[i] = (float) in[i]
-void to_float(const LaCtx& la, const double* in, long long n, float* out, double scale = 1.0);
 
 // Mirror the lower triangle into the upper one for each of `batch` n x n slices.
 void symmetrize_lower(const LaCtx& la, double* X, int n, int batch);

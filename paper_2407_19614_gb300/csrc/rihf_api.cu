@@ -966,7 +966,7 @@ static void compute_geometry_rest(rihf_ctx* c) {
     dgemm(la, g1);
     GemmArgs g2;   // T2 (n x n) = -1/2 X^T T1, then + 3/2 I
     g2.M = nind; g2.N = nind; g2.K = N; g2.A = c->Xo; g2.lda = nind; g2.transA = true; g2.B = c->T1;
-    g2.ldb = nind; g2.C = c->T2; g2.ldc = nind; g2.alpha = -0.5;
+    g2.ldb = nind; g2.C = c->T2; g2.ldc = nind; g2.alpha = -0.5; g2.lower_only = g2.mirror = true;
     dgemm(la, g2);
     identity(la, c->Err, nind);
     axpby(la, nind * nind, 1.0, c->T2, 1.5, c->Err, c->T2);
@@ -1346,7 +1346,7 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
     dgemm(la, g1);
     GemmArgs g2;   // Fp (n x n) = Xo^T T1
     g2.M = n; g2.N = n; g2.K = N; g2.A = c->Xo; g2.lda = n; g2.transA = true; g2.B = c->T1; g2.ldb = n;
-    g2.C = c->Fp; g2.ldc = n;
+    g2.C = c->Fp; g2.ldc = n; g2.lower_only = g2.mirror = true;
     dgemm(la, g2);
     RIHF_CUDA(cudaMemsetAsync(c->eps, 0, sizeof(double) * N, c->stream));
   };
@@ -1380,7 +1380,7 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
       // guard: orthonormality and the off-diagonal of Cp^T F' Cp
       GemmArgs go;   // T2 = Cp^T Cp
       go.M = n; go.N = n; go.K = n; go.A = c->Cp; go.lda = n; go.transA = true; go.B = c->Cp; go.ldb = n;
-      go.C = c->T2; go.ldc = n;
+      go.C = c->T2; go.ldc = n; go.lower_only = go.mirror = true;
       dgemm(la, go);
       eig_check_mb_kernel<<<kRedBlocks, 256, 0, c->stream>>>(c->T2, n, 1.0, 0, c->d_red, c->d_ticket, c->scal + 2);
       RIHF_LAUNCH_CHECK();
@@ -1389,7 +1389,7 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
       dgemm(la, gf);
       GemmArgs gt;
       gt.M = n; gt.N = n; gt.K = n; gt.A = c->Cp; gt.lda = n; gt.transA = true; gt.B = c->T1; gt.ldb = n;
-      gt.C = c->T2; gt.ldc = n;
+      gt.C = c->T2; gt.ldc = n; gt.lower_only = gt.mirror = true;
       dgemm(la, gt);
       // occupied-virtual block only: rotations inside the occupied or the
       // virtual space (near-degenerate pairs) leave the density unchanged
@@ -1522,7 +1522,7 @@ static void fock_build(rihf_ctx* c) {
   form_Ct(c);
   GemmArgs gd;
   gd.M = N; gd.N = N; gd.K = no; gd.A = c->Ct; gd.lda = no; gd.B = c->Ct; gd.ldb = no; gd.transB = true;
-  gd.C = c->D; gd.ldc = N;
+  gd.C = c->D; gd.ldc = N; gd.lower_only = gd.mirror = true;
   dgemm(la, gd);
   ri_j(c);
   // RI-K: Hb[P] = B^P Ct (N x nocc); K = -1/2 sum_P Hb[P] Hb[P]^T
@@ -1531,10 +1531,9 @@ static void fock_build(rihf_ctx* c) {
   gk.M = N; gk.N = N; gk.K = no; gk.A = c->Hb; gk.lda = no; gk.sA = (long long)N * no;
   gk.B = c->Hb; gk.ldb = no; gk.sB = (long long)N * no; gk.transB = true;
   gk.C = c->K; gk.ldc = N; gk.batch = NA; gk.reduce_batch = true; gk.alpha = -0.5;
-  gk.lower_only = true;   // K is symmetric: lower tiles only, then mirror
+  gk.lower_only = gk.mirror = true;   // K is symmetric
   { TraceScope t(c->tracer, c->stream, "RI-K K=-1/2 sum H H^T (dgemm)", 2.0 * NA * n2 * no, 0);
-    dgemm(la, gk);
-    symmetrize_lower(la, c->K, N, 1); }
+    dgemm(la, gk); }
   add3(la, (int)n2, c->H, c->J, c->K, c->F);
   if (c->sph_avg) {
     sph_avg_kernel<<<std::max(1, std::min(ceil_div((long long)n2, 256), 8 * c->sms)), 256, 0, c->stream>>>(
@@ -1623,7 +1622,7 @@ static void fock_build_tc(rihf_ctx* c, int digits) {
   form_Ct(c);
   GemmArgs gd;
   gd.M = N; gd.N = N; gd.K = no; gd.A = c->Ct; gd.lda = no; gd.B = c->Ct; gd.ldb = no; gd.transB = true;
-  gd.C = c->D; gd.ldc = N;
+  gd.C = c->D; gd.ldc = N; gd.lower_only = gd.mirror = true;
   dgemm(la, gd);
   ri_j(c);
   const double prod = oz_products(digits);
@@ -2110,7 +2109,7 @@ static void fock_build_factor(rihf_ctx* c, int variant) {
   cudaStream_t s = c->stream;
   GemmArgs gd;
   gd.M = N; gd.N = N; gd.K = m; gd.A = c->d_sad; gd.lda = m; gd.B = c->d_sad; gd.ldb = m; gd.transB = true;
-  gd.C = c->D; gd.ldc = N;
+  gd.C = c->D; gd.ldc = N; gd.lower_only = gd.mirror = true;
   dgemm(la, gd);
   ri_j(c);
   for (int c0 = 0; c0 < m; c0 += no) {
@@ -2192,7 +2191,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
       // Cprev^T = L^{-1} V^T; large nuclear steps leave V far from orthonormal
       GemmArgs m3;   // Cprev = T2^T T2
       m3.M = n; m3.N = n; m3.K = n; m3.A = c->T2; m3.lda = n; m3.transA = true; m3.B = c->T2; m3.ldb = n;
-      m3.C = c->Cprev; m3.ldc = n;
+      m3.C = c->Cprev; m3.ldc = n; m3.lower_only = m3.mirror = true;
       dgemm(la, m3);
       RIHF_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
       cholesky(la, c->Cprev, n, c->scratch);
@@ -2252,7 +2251,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     dgemm(la, g1);
     GemmArgs g2;   // T2 (no x no) = Co^T T1
     g2.M = no; g2.N = no; g2.K = N; g2.A = c->Ct; g2.lda = no; g2.transA = true; g2.B = c->T1; g2.ldb = no;
-    g2.C = c->T2; g2.ldc = no;
+    g2.C = c->T2; g2.ldc = no; g2.lower_only = g2.mirror = true;
     dgemm(la, g2);
     cholesky(la, c->T2, no, c->scratch);
     transpose(la, c->Ct, N, no, c->T1);                        // T1 = Co^T (no x N)
@@ -2440,7 +2439,7 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   form_Ct(c);
   GemmArgs gd;
   gd.M = N; gd.N = N; gd.K = no; gd.A = c->Ct; gd.lda = no; gd.B = c->Ct; gd.ldb = no; gd.transB = true;
-  gd.C = c->D; gd.ldc = N;
+  gd.C = c->D; gd.ldc = N; gd.lower_only = gd.mirror = true;
   dgemm(la, gd);
   // W = 2 sum_i eps_i C_i C_i^T = 1/2 D F D at convergence (C~^T F C~ = 2 diag(eps_occ));
   // this form needs no individual eigenvectors inside near-degenerate clusters
@@ -2449,7 +2448,7 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   dgemm(la, gf);
   GemmArgs gw;
   gw.M = N; gw.N = N; gw.K = N; gw.A = c->D; gw.lda = N; gw.B = c->T2; gw.ldb = N; gw.C = c->W; gw.ldc = N;
-  gw.alpha = 0.5;
+  gw.alpha = 0.5; gw.lower_only = gw.mirror = true;
   dgemm(la, gw);
   // d = B vec D; c = L^{-T} d (the paper's L^P) is solved below together with X~
   { TraceScope t(c->tracer, s, "grad d = B D (gemv over packed rows)", (double)NA * c->npp * 8, 1);
