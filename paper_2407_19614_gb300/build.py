@@ -19,7 +19,7 @@ SRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librihf.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["rihf_api.cu", "grad_eri3_lane.cu", "eri3_lane.cu", "integrals.cu", "grad_integrals.cu", "linalg.cu", "eigh_tridiag.cu", "jk.cu", "eigh_noalloc.cu", "tc_gemm.cu", "mlp.cu"]
+SOURCES = ["rihf_api.cu", "grad_eri3_lane.cu", "grad_one_lane.cu", "eri3_lane.cu", "one_lane.cu", "eri2_lane.cu", "integrals.cu", "grad_integrals.cu", "linalg.cu", "eigh_tridiag.cu", "jk.cu", "eigh_noalloc.cu", "tc_gemm.cu", "mlp.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -274,7 +274,7 @@ __device__ __forceinline__ void lane_hrr(const double* k, const double (&AB)[3],
 // ------------------------------------------------------------ bra solid harmonics
 
 // Coefficient of Cartesian component (x, y, z) in the real solid harmonic m of
-// degree l <= 3, every function with the norm of x^l (the library's rows of the
+// degree l <= 4, every function with the norm of x^l (the library's rows of the
 // transform table, spelt out so that the zeros cost nothing).
 __host__ __device__ constexpr double bra_sph(int l, int m, int x, int y, int z) {
   if (l == 0) return 1.0;
@@ -287,6 +287,20 @@ __host__ __device__ constexpr double bra_sph(int l, int m, int x, int y, int z) 
     if (m == 0) return z == 2 ? 1.0 : (x == 2 || y == 2 ? -0.5 : 0.0);
     if (m == 1) return x == 1 && z == 1 ? s3 : 0.0;
     return x == 2 ? 0.5 * s3 : (y == 2 ? -0.5 * s3 : 0.0);
+  }
+  if (l == 4) {
+    constexpr double s5 = 2.2360679774997896964, s35 = 5.9160797830996160426, s70 = 8.3666002653407554798;
+    if (m == -4) return x == 3 && y == 1 ? 0.5 * s35 : (x == 1 && y == 3 ? -0.5 * s35 : 0.0);
+    if (m == -3) return z == 1 && x == 2 ? 0.75 * s70 : (z == 1 && y == 3 ? -0.25 * s70 : 0.0);
+    if (m == -2) return x == 1 && y == 1 ? 3.0 * s5 : ((x == 3 && y == 1) || (x == 1 && y == 3) ? -0.5 * s5 : 0.0);
+    if (m == -1) return y == 1 && z == 3 ? 4.0 * s58 : (z == 1 && (y == 3 || (x == 2 && y == 1)) ? -3.0 * s58 : 0.0);
+    if (m == 0)
+      return z == 4 ? 1.0 : (z == 2 ? (x == 2 || y == 2 ? -3.0 : 0.0) : (z == 0 ? (x == 2 ? 0.75 : (x == 4 || y == 4 ? 0.375 : 0.0)) : 0.0));
+    if (m == 1) return x == 1 && z == 3 ? 4.0 * s58 : (z == 1 && (x == 3 || (x == 1 && y == 2)) ? -3.0 * s58 : 0.0);
+    if (m == 2)
+      return z == 2 ? (x == 2 ? 1.5 * s5 : (y == 2 ? -1.5 * s5 : 0.0)) : (x == 4 ? -0.25 * s5 : (y == 4 ? 0.25 * s5 : 0.0));
+    if (m == 3) return z == 1 && x == 3 ? 0.25 * s70 : (z == 1 && x == 1 && y == 2 ? -0.75 * s70 : 0.0);
+    return x == 4 || y == 4 ? 0.125 * s35 : (x == 2 && y == 2 ? -0.75 * s35 : 0.0);
   }
   if (m == -3) return x == 2 && y == 1 ? 3.0 * s58 : (y == 3 ? -s58 : 0.0);
   if (m == -2) return x == 1 && y == 1 && z == 1 ? s15 : 0.0;

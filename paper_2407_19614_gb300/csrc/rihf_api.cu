@@ -18,6 +18,7 @@
 #include "eri3_lane.cuh"
 #include "integrals.cuh"
 #include "jk.cuh"
+#include "lane2.cuh"
 #include "linalg.cuh"
 #include "os_hgp.cuh"
 #include "mlp.cuh"
@@ -500,6 +501,9 @@ struct rihf_ctx {
   LaneChunk* d_chunks = nullptr;     // its chunk lists
   size_t chunk_cap = 0;
   KetTable* d_ket = nullptr;
+  Lane2Tasks lane_eri2, lane_one;    // (P|Q) and one-electron shell pairs, of the basis alone
+  int2* d_tasks2 = nullptr;
+  LaneChunk* d_chunks2 = nullptr;
   double* d_schwarz = nullptr;
   bool schwarz_ok = false;
   bool schwarz_fresh = false;   // d_schwarz holds Q of the current geometry
@@ -742,7 +746,7 @@ static void free_all(rihf_ctx* c) {
                   c->d_ao_atom, c->d_ao_l, c->hist_D[0], c->hist_D[1], c->hist_D[2], c->hist_S, c->hist_xyz[0],
                   c->hist_xyz[1], c->Shalf, c->Smhalf, c->DL, c->Dpred, c->mlX, c->mly, c->mlt, c->mlDx, c->ml_sums, c->rep_X, c->rep_t, c->net.master, c->net.wbf, c->net.grad,
                   c->net.m, c->net.v, c->net.loss,
-                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_flag, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_chunks, c->d_ket, c->d_schwarz,
+                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_flag, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_chunks, c->d_ket, c->d_tasks2, c->d_chunks2, c->d_schwarz,
                   c->S, c->H, c->Tk, c->V, c->A, c->L, c->Linv, c->Bp, c->Yp, c->Bu, c->Dp, c->Jp, c->Xo, c->Sw, c->Sv,
                   c->C, c->eps, c->Ct, c->D, c->J, c->K, c->F, c->Fx, c->T1, c->T2, c->Err, c->Fp, c->Cp, c->Hb,
                   c->dvec, c->Fring, c->Ering, c->Bdiis, c->coef, c->scal, c->Cprev,
@@ -809,11 +813,16 @@ static void compute_geometry(rihf_ctx* c, bool defer_eri3 = false) {
   cudaEventRecord(c->ev[0], s);
   DevShells P = c->prim(), X = c->aux();
   { TraceScope t(c->tracer, s, "one_electron_kernel (S,T,V)", 3.0 * N * N * 8, 1);
-    launch_one_electron(ic, P, c->max_lp, c->natoms, c->d_Z, c->d_xyz, c->S, c->Tk, c->V); }
-  axpby(la, N * N, 1.0, c->Tk, 1.0, c->V, c->H);
+    if (c->opt.pure) {
+      launch_lane_one(ic, P, c->lane_one, c->natoms, c->d_Z, c->d_xyz, c->S, c->H);
+    } else {
+      launch_one_electron(ic, P, c->max_lp, c->natoms, c->d_Z, c->d_xyz, c->S, c->Tk, c->V);
+      axpby(la, N * N, 1.0, c->Tk, 1.0, c->V, c->H);
+    } }
   // metric, Cholesky, L^{-1}
   { TraceScope t(c->tracer, s, "eri2_kernel (P|Q)", (double)NA * NA * 8, 1);
-    launch_eri2(ic, X, c->max_la, c->A); }
+    if (c->opt.pure) launch_lane_eri2(ic, X, c->lane_eri2, c->d_ket, c->A);
+    else launch_eri2(ic, X, c->max_la, c->A); }
   RIHF_CUDA(cudaMemcpyAsync(c->L, c->A, sizeof(double) * NA * NA, cudaMemcpyDeviceToDevice, s));
   { TraceScope t(c->tracer, s, "cholesky A=LL^T", (double)NA * NA * NA / 3.0, 0);
     cholesky(la, c->L, NA, c->scratch); }
@@ -1122,6 +1131,21 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       c->d_ket = dalloc<KetTable>(ket.size());
       upload(c->d_ket, ket, s);
       RIHF_CUDA(cudaStreamSynchronize(s));
+    }
+    if (c->opt.pure) {   // the task lists of the two-centre and one-electron kernels, of the basis alone
+      std::vector<int2> t2, t1;
+      std::vector<LaneChunk> c2, c1;
+      build_lane2_tasks(c->ha.l, c->ha.atom, t2, c2);
+      build_one_tasks(c->hp.l, t1, c1);
+      c->d_tasks2 = dalloc<int2>(t2.size() + t1.size());
+      c->d_chunks2 = dalloc<LaneChunk>(c2.size() + c1.size());
+      upload(c->d_tasks2, t2, s);
+      upload(c->d_tasks2 + t2.size(), t1, s);
+      upload(c->d_chunks2, c2, s);
+      upload(c->d_chunks2 + c2.size(), c1, s);
+      RIHF_CUDA(cudaStreamSynchronize(s));   // the host lists are temporaries
+      c->lane_eri2 = {c->d_tasks2, c->d_chunks2, (long long)c2.size()};
+      c->lane_one = {c->d_tasks2 + t2.size(), c->d_chunks2 + c2.size(), (long long)c1.size()};
     }
     refresh_tasks(c);
     {
@@ -2591,14 +2615,18 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   double* g_three = c->grad_parts + 6 * nat;
   double* g_two = c->grad_parts + 9 * nat;
   { TraceScope t(c->tracer, s, "grad_one_electron_kernel", 0.0, 0);
-    launch_grad_one_electron(ic, c->prim(), c->max_lp, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl); }
+    if (c->opt.pure)
+      launch_lane_grad_one(ic, c->prim(), c->lane_one, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl);
+    else
+      launch_grad_one_electron(ic, c->prim(), c->max_lp, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl); }
   if (!defer_eri3) {
     TraceScope t(c->tracer, s, "grad_eri3_kernel (fused d(mu nu|P) . Y)", c->flops_grad3, 0);
     if (c->opt.pure) launch_lane_grad(ic, c->sms, lane_tasks(c, g_three, c->Yp));
     else launch_grad_eri3(ic, c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, c->Yp, g_three);
   }
   { TraceScope t(c->tracer, s, "grad_eri2_kernel (fused d(P|Q) . Z)", (double)NA * NA * 8, 1);
-    launch_grad_eri2(ic, c->aux(), c->max_la, c->Zm, g_two); }
+    if (c->opt.pure) launch_lane_grad_eri2(ic, c->aux(), c->lane_eri2, c->d_ket, c->Zm, g_two);
+    else launch_grad_eri2(ic, c->aux(), c->max_la, c->Zm, g_two); }
 }
 
 // Per-atom parts back to the host, nuclear repulsion, the sum.

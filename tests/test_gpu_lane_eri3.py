@@ -1,6 +1,6 @@
-"""The one-lane-per-task 3-centre kernels at the edges of their classes and ranges, against the oracle.
+"""The one-lane-per-task integral kernels at the edges of their classes and ranges, against the oracle.
 
-T3 element-wise to 1e-12 of its largest element (the bound of the other integral tests: sums of a
+Integrals element-wise to 1e-12 of the largest element (the bound of the other integral tests: sums of a
 few hundred FP64 terms, each a few rounding units).  Gradients to the 1e-8 Eh/bohr of the other
 parity tests, in a basis whose overlap is well conditioned: an orbital error e moves the forces by
 about e / (gap sqrt(lambda_min(S))), so SCF errors of 1e-9 stay below 1e-8 at lambda_min 0.017 (the
@@ -81,6 +81,17 @@ def test_three_centre_integrals(name):
     T = ctx.matrix("T3")
     ctx.close()
     assert np.abs(T - s.T3).max() <= 1e-12 * np.abs(s.T3).max()
+
+
+@pytest.mark.parametrize("name", ["small shuffled", "f and g shuffled", "mixed contraction", "far, f and g"])
+def test_metric_and_one_electron(name):
+    R = _R()
+    mol = _case(name)
+    s = O.System(mol)
+    ctx = R.Context(mol)
+    for what, ref in (("A", s.A), ("S", s.S), ("H", s.h)):
+        assert np.abs(ctx.matrix(what) - ref).max() <= 1e-12 * np.abs(ref).max(), what
+    ctx.close()
 
 
 @pytest.mark.parametrize("name", ["small shuffled", "f and g conditioned", "mixed contraction conditioned",
