@@ -626,128 +626,54 @@ void trsm_lower_t_tc(const LaCtx& la, const double* L, int n, double* X, long lo
 
 // ------------------------------------------------------------ eigensolver
 
-constexpr int JT = 1024;   // Jacobi threads (one CTA)
-constexpr int kJRows = 8;  // rows per lane of the register-resident one-sided Jacobi (n <= 256)
+// One-sided (Hestenes) Jacobi in FP32: with B = A + sigma I positive definite
+// (sigma from a Gershgorin bound), column rotations U <- U J drive the columns of
+// U = B V to mutual orthogonality; then v_j = u_j / |u_j| and lambda_j = |u_j| -
+// sigma.  Only U (n x n, column-major) is stored.
+//
+// The columns form nb blocks of H (nb even); in a round a warp holds the two
+// blocks of one block pair in registers (R rows of every column per lane) and
+// rotates every column pair across them (round 0 also the pairs inside each
+// block); a sweep is the nb - 1 rounds of the round-robin order.  Squared column
+// norms are carried by the rotation identities |u_p'|^2 = |u_p|^2 - t (u_p . u_q),
+// |u_q'|^2 = |u_q|^2 + t (u_p . u_q) and recomputed at every sweep, so a pair costs
+// one reduction.  The H rotations of one step are independent and written without
+// branches, so that their reductions overlap.
+//
+// What bounds it is the latency of a round, so that a single CTA with all 32 warps
+// of a 192 x 192 problem on one SM was bound by that SM's issue slots and shared
+// memory (0.45 ms a sweep).  Above n = 64 the pairs are spread over a cluster of
+// CL = 8 CTAs, the columns pass through L2 (.cg loads and stores) and a cluster
+// barrier ends each round: 0.24 ms a sweep.  Up to n = 64 one CTA with U in shared
+// memory is faster than the barrier (n = 24: 81 us to convergence, 104 us when its
+// rounds ran over 64 mostly empty blocks).
+constexpr int kJacobiCluster = 8;
+constexpr int kJacobiSmall = 64;
 
-// Parallel cyclic Jacobi (round-robin pairing) in FP32, one CTA.  a: m x m
-// working matrix (shared or global), v: n x m eigenvector matrix (global).
-__device__ void jacobi_f32(float* a, float* v, int n, int m, int max_sweeps, float* cs, float* sn, float* tt,
-                           int* pp, int* qq, float* red) {
-  const int tid = threadIdx.x;
-  const int half = m / 2;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    // convergence test: off-diagonal vs diagonal Frobenius mass
-    float off = 0.f, dia = 0.f;
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int i = warp; i < m; i += JT / 32)
-      for (int j = lane; j < m; j += 32) {
-        float x = a[i * m + j];
-        if (i == j) dia += x * x; else off += x * x;
-      }
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      dia += __shfl_xor_sync(0xffffffffu, dia, o);
-    }
-    if ((tid & 31) == 0) { red[tid / 32] = off; red[32 + tid / 32] = dia; }
-    __syncthreads();
-    if (tid == 0) {
-      float so = 0.f, sd = 0.f;
-      for (int w = 0; w < JT / 32; ++w) { so += red[w]; sd += red[32 + w]; }
-      red[64] = so;
-      red[65] = sd;
-    }
-    __syncthreads();
-    float so = red[64], sd = red[65];
-    __syncthreads();
-    // FP32 stops near its rounding floor; the FP64 refinement takes over
-    if (so <= 1e-10f * sd || so == 0.f) break;
-    for (int r = 0; r < m - 1; ++r) {
-      // pairs: (m-1, r) and ((r+k) mod (m-1), (r-k) mod (m-1)), k = 1..half-1
-      for (int k = tid; k < half; k += JT) {
-        int p, q;
-        if (k == 0) { p = r; q = m - 1; }
-        else { p = (r + k) % (m - 1); q = (r - k + (m - 1)) % (m - 1); }
-        if (p > q) { int t = p; p = q; q = t; }
-        float apq = a[p * m + q], app = a[p * m + p], aqq = a[q * m + q];
-        float c = 1.f, s = 0.f, t = 0.f;
-        if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-9f * sqrtf(fabsf(app * aqq))) {
-          float tau = (aqq - app) / (2.f * apq);
-          t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-          c = rsqrtf(1.f + t * t);
-          s = t * c;
-        }
-        pp[k] = p; qq[k] = q; cs[k] = c; sn[k] = s; tt[k] = t;
-      }
-      __syncthreads();
-      // two-sided update of all 2x2 blocks (k1, k2): warp per k1, lane per k2
-      for (int k1 = warp; k1 < half; k1 += JT / 32) {
-        const int p1 = pp[k1], q1 = qq[k1];
-        const float c1 = cs[k1], s1 = sn[k1];
-        for (int k2 = lane; k2 < half; k2 += 32) {
-          const int p2 = pp[k2], q2 = qq[k2];
-          if (k1 == k2) {
-            float apq = a[p1 * m + q1];
-            a[p1 * m + p1] -= tt[k1] * apq;
-            a[q1 * m + q1] += tt[k1] * apq;
-            a[p1 * m + q1] = 0.f;
-            a[q1 * m + p1] = 0.f;
-            continue;
-          }
-          const float c2 = cs[k2], s2 = sn[k2];
-          float app = a[p1 * m + p2], apq = a[p1 * m + q2], aqp = a[q1 * m + p2], aqq = a[q1 * m + q2];
-          // right rotation (columns p2, q2)
-          float xp = c2 * app - s2 * apq, xq = s2 * app + c2 * apq;
-          float yp = c2 * aqp - s2 * aqq, yq = s2 * aqp + c2 * aqq;
-          // left rotation (rows p1, q1)
-          a[p1 * m + p2] = c1 * xp - s1 * yp;
-          a[p1 * m + q2] = c1 * xq - s1 * yq;
-          a[q1 * m + p2] = s1 * xp + c1 * yp;
-          a[q1 * m + q2] = s1 * xq + c1 * yq;
-        }
-      }
-      // eigenvectors: V <- V J
-      for (int i = warp; i < n; i += JT / 32)
-        for (int k = lane; k < half; k += 32) {
-          int p = pp[k], q = qq[k];
-          float c = cs[k], s = sn[k];
-          float vp = v[i * m + p], vq = v[i * m + q];
-          v[i * m + p] = c * vp - s * vq;
-          v[i * m + q] = s * vp + c * vq;
-        }
-      __syncthreads();
-    }
-  }
-}
-
-__global__ void __launch_bounds__(JT) jacobi_kernel(const double* __restrict__ A, int n, int m, float* gA,
-                                                    float* V, float* W, int use_smem, int max_sweeps) {
+template <int H, int R, int CL>
+__global__ void __launch_bounds__(CL == 1 ? 1024 : 32 * 4)
+    jacobi1s_kernel(const double* __restrict__ A, int n, int m, float* gU, float* __restrict__ V, float* W, int nb,
+                    int max_sweeps, float tol) {
+  namespace cg = cooperative_groups;
   extern __shared__ float sm[];
-  __shared__ float cs[1024], sn[1024], tt[1024];
-  __shared__ int pp[1024], qq[1024];
-  __shared__ float red[72];
-  float* a = use_smem ? sm : gA;
-  for (int idx = threadIdx.x; idx < m * m; idx += JT) {
-    int i = idx / m, j = idx % m;
-    a[idx] = (i < n && j < n) ? (float)A[(size_t)i * n + j] : 0.f;
-  }
-  for (int idx = threadIdx.x; idx < n * m; idx += JT) {
-    int i = idx / m, j = idx % m;
-    V[idx] = (i == j) ? 1.f : 0.f;
-  }
-  __syncthreads();
-  jacobi_f32(a, V, n, m, max_sweeps, cs, sn, tt, pp, qq, red);
-  __syncthreads();
-  for (int i = threadIdx.x; i < m; i += JT) W[i] = a[i * m + i];
-}
-
-constexpr int kJB = 64;   // column blocks of the block one-sided Jacobi (two per warp)
-
-// U (column-major, n x n) = A + sigma I with the Gershgorin shift sigma =
-// 1.05 max_i sum_j |A_ij|, which makes the matrix positive definite.
-__device__ float jacobi_shifted_copy(const double* __restrict__ A, int n, float* U, float* red) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ float red[33];
+  __shared__ int flag;   // a pair was rotated in this sweep
+  const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = CL == 1 ? 0 : (int)blockIdx.x, gw = rank * warps + warp, nw = CL * warps;   // warp of the cluster
+  float* U = CL == 1 ? sm : gU;
+  auto sync = [&]() {
+    if constexpr (CL == 1) __syncthreads();
+    else cg::this_cluster().sync();
+  };
+  auto ld = [&](const float* x) -> float { return CL == 1 ? *x : __ldcg(x); };
+  auto st = [&](float* x, float v) {
+    if constexpr (CL == 1) *x = v;
+    else __stcg(x, v);
+  };
+  const float tol2 = tol * tol;
+  // sigma = 1.05 max_i sum_j |A_ij|
   float g = 0.f;
-  for (int i = warp; i < n; i += JT / 32) {
+  for (int i = gw; i < n; i += nw) {
     float s = 0.f;
     for (int j = lane; j < n; j += 32) s += fabsf((float)A[(size_t)i * n + j]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -755,250 +681,148 @@ __device__ float jacobi_shifted_copy(const double* __restrict__ A, int n, float*
   }
   if (lane == 0) red[warp] = g;
   __syncthreads();
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     float t = 0.f;
-    for (int w = 0; w < JT / 32; ++w) t = fmaxf(t, red[w]);
-    red[0] = 1.05f * t + 1e-20f;
+    for (int w = 0; w < warps; ++w) t = fmaxf(t, red[w]);
+    red[32] = t;
   }
-  __syncthreads();
-  const float sigma = red[0];
-  for (int j = warp; j < n; j += JT / 32)
-    for (int i = lane; i < n; i += 32) U[(size_t)j * n + i] = (float)A[(size_t)i * n + j] + (i == j ? sigma : 0.f);
-  __syncthreads();
-  return sigma;
-}
-
-// Eigenpairs of the orthogonalised columns: v_j = u_j / |u_j|, lambda_j =
-// |u_j| - sigma; V row-major n x m.
-__device__ void jacobi_eigenpairs(const float* U, int n, int m, float sigma, float* V, float* W) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int j = warp; j < n; j += JT / 32) {
+  sync();
+  float top = red[32];
+  if constexpr (CL > 1)
+    for (int q = 0; q < CL; ++q) top = fmaxf(top, *cg::this_cluster().map_shared_rank(red + 32, q));
+  const float sigma = 1.05f * top + 1e-20f;
+  for (int j = gw; j < n; j += nw)
+    for (int i = lane; i < n; i += 32) st(U + (size_t)j * n + i, (float)A[(size_t)i * n + j] + (i == j ? sigma : 0.f));
+  sync();
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    if (threadIdx.x == 0) flag = 0;
+    // squared norms, kept in W until the end
+    for (int j = gw; j < n; j += nw) {
+      const float* u = U + (size_t)j * n;
+      float s2 = 0.f;
+      for (int i = lane; i < n; i += 32) {
+        const float x = ld(u + i);
+        s2 = fmaf(x, x, s2);
+      }
+      for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      if (lane == 0) __stcg(W + j, s2);
+    }
+    sync();
+    bool rotated = false;
+    for (int r = 0; r < nb - 1; ++r) {
+      if (gw < nb / 2) {
+        const int bA = gw == 0 ? nb - 1 : (r + gw) % (nb - 1), bB = gw == 0 ? r : (r - gw + nb - 1) % (nb - 1);
+        float x[2 * H][R], cn[2 * H];
+#pragma unroll
+        for (int c = 0; c < 2 * H; ++c) {
+          const int col = c < H ? bA * H + c : bB * H + c - H;
+          cn[c] = col < n ? __ldcg(W + col) : 0.f;
+#pragma unroll
+          for (int e = 0; e < R; ++e) {
+            const int i = lane + 32 * e;
+            x[c][e] = col < n && i < n ? ld(U + (size_t)col * n + i) : 0.f;
+          }
+        }
+        auto rot = [&](float (&xp)[R], float (&xq)[R], float& a, float& b) {
+          float c = 0.f;
+#pragma unroll
+          for (int e = 0; e < R; ++e) c = fmaf(xp[e], xq[e], c);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+          // fast divisions and roots: the angle needs a few digits only, and c^2 + s^2 = 1
+          // holds to the rounding of rsqrtf
+          const bool act = c * c > (tol2 * a) * b;   // not a converged pair, nor a zero (padding) column
+          rotated |= act;
+          const float zeta = fminf(fmaxf(__fdividef(b - a, 2.f * (act ? c : 1.f)), -1e18f), 1e18f);
+          const float z2 = fmaf(zeta, zeta, 1.f);
+          const float t = act ? copysignf(__fdividef(1.f, fabsf(zeta) + z2 * rsqrtf(z2)), zeta) : 0.f;
+          const float cs = act ? rsqrtf(fmaf(t, t, 1.f)) : 1.f, sn = cs * t;
+#pragma unroll
+          for (int e = 0; e < R; ++e) {
+            const float u = xp[e], v = xq[e];
+            xp[e] = cs * u - sn * v;
+            xq[e] = sn * u + cs * v;
+          }
+          a -= t * c;
+          b += t * c;
+        };
+        if (r == 0) {
+#pragma unroll
+          for (int p = 0; p < H; ++p)
+#pragma unroll
+            for (int q = p + 1; q < H; ++q) {
+              rot(x[p], x[q], cn[p], cn[q]);
+              rot(x[H + p], x[H + q], cn[H + p], cn[H + q]);
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < H; ++d)
+#pragma unroll
+          for (int p = 0; p < H; ++p) rot(x[p], x[H + (p + d) % H], cn[p], cn[H + (p + d) % H]);
+#pragma unroll
+        for (int c = 0; c < 2 * H; ++c) {
+          const int col = c < H ? bA * H + c : bB * H + c - H;
+          if (col < n) {
+#pragma unroll
+            for (int e = 0; e < R; ++e) {
+              const int i = lane + 32 * e;
+              if (i < n) st(U + (size_t)col * n + i, x[c][e]);
+            }
+            if (lane == 0) __stcg(W + col, cn[c]);
+          }
+        }
+      }
+      sync();
+    }
+    if (rotated && lane == 0) flag = 1;
+    sync();
+    bool more = flag != 0;
+    if constexpr (CL > 1)
+      for (int q = 0; q < CL; ++q) more |= *cg::this_cluster().map_shared_rank(&flag, q) != 0;
+    sync();   // every flag has been read
+    if (!more) break;
+  }
+  // eigenpairs of the orthogonalised columns; V row-major n x m
+  for (int j = gw; j < n; j += nw) {
     const float* u = U + (size_t)j * n;
     float s = 0.f;
-    for (int i = lane; i < n; i += 32) s = fmaf(u[i], u[i], s);
+    for (int i = lane; i < n; i += 32) {
+      const float x = ld(u + i);
+      s = fmaf(x, x, s);
+    }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    float nrm = sqrtf(s);
-    float inv = nrm > 0.f ? 1.f / nrm : 0.f;
-    for (int i = lane; i < n; i += 32) V[(size_t)i * m + j] = u[i] * inv;
+    const float nrm = sqrtf(s), inv = nrm > 0.f ? 1.f / nrm : 0.f;
+    for (int i = lane; i < n; i += 32) V[(size_t)i * m + j] = ld(u + i) * inv;
     if (lane == 0) W[j] = nrm - sigma;
   }
 }
 
-// One-sided (Hestenes) Jacobi in FP32, one CTA: with B = A + sigma I positive
-// definite (sigma from a Gershgorin bound), column rotations U <- U J drive the
-// columns of U = B V to mutual orthogonality; then v_j = u_j / |u_j| and
-// lambda_j = |u_j| - sigma.  Only U (n x n, column-major, shared memory when it
-// fits) is stored; a warp owns one column pair per round (round-robin pairing),
-// its dot products reduced with shuffles.  For n <= 256 a pair's columns stay
-// in registers between the dot product and the rotation, and the squared
-// column norms are carried along by the rotation identities
-// |u_p'|^2 = |u_p|^2 - t (u_p . u_q), |u_q'|^2 = |u_q|^2 + t (u_p . u_q)
-// (recomputed at every sweep), so a pair costs one reduction, not three.
-__global__ void __launch_bounds__(JT) jacobi1s_kernel(const double* __restrict__ A, int n, int m, float* gU, float* V,
-                                                      float* W, int use_smem, int max_sweeps, float tol) {
-  extern __shared__ float sm[];
-  __shared__ float red[32];
-  __shared__ float nrm[32 * kJRows];
-  __shared__ int notconv;
-  float* U = use_smem ? sm : gU;   // column j at U[j*n .. j*n+n)
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float sigma = jacobi_shifted_copy(A, n, U, red);
-  const int half = m / 2;
-  const bool in_regs = n <= 32 * kJRows;
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) notconv = 0;
-    if (in_regs) {
-      for (int j = warp; j < n; j += JT / 32) {
-        const float* u = U + (size_t)j * n;
-        float s2 = 0.f;
-        for (int i = lane; i < n; i += 32) s2 = fmaf(u[i], u[i], s2);
-        for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        if (lane == 0) nrm[j] = s2;
-      }
-    }
-    __syncthreads();
-    for (int r = 0; r < m - 1 && in_regs; ++r) {
-      for (int k = warp; k < half; k += JT / 32) {
-        int p, q;
-        if (k == 0) { p = r; q = m - 1; }
-        else { p = (r + k) % (m - 1); q = (r - k + (m - 1)) % (m - 1); }
-        if (p >= n || q >= n) continue;   // padding column
-        float* up = U + (size_t)p * n;
-        float* uq = U + (size_t)q * n;
-        float x[kJRows], y[kJRows];
-        float c = 0.f;
-#pragma unroll
-        for (int e = 0; e < kJRows; ++e) {
-          const int i = lane + 32 * e;
-          x[e] = i < n ? up[i] : 0.f;
-          y[e] = i < n ? uq[i] : 0.f;
-          c = fmaf(x[e], y[e], c);
-        }
-        const float a = nrm[p], b = nrm[q];
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (fabsf(c) <= tol * sqrtf(a * b)) continue;
-        if (lane == 0) notconv = 1;
-        float zeta = (b - a) / (2.f * c);
-        float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-        float cs = rsqrtf(1.f + t * t), sn = cs * t;
-#pragma unroll
-        for (int e = 0; e < kJRows; ++e) {
-          const int i = lane + 32 * e;
-          if (i < n) {
-            up[i] = cs * x[e] - sn * y[e];
-            uq[i] = sn * x[e] + cs * y[e];
-          }
-        }
-        if (lane == 0) {
-          nrm[p] = a - t * c;
-          nrm[q] = b + t * c;
-        }
-      }
-      __syncthreads();
-    }
-    for (int r = 0; r < m - 1 && !in_regs; ++r) {
-      for (int k = warp; k < half; k += JT / 32) {
-        int p, q;
-        if (k == 0) { p = r; q = m - 1; }
-        else { p = (r + k) % (m - 1); q = (r - k + (m - 1)) % (m - 1); }
-        if (p >= n || q >= n) continue;   // padding column
-        float* up = U + (size_t)p * n;
-        float* uq = U + (size_t)q * n;
-        float a = 0.f, b = 0.f, c = 0.f;
-        for (int i = lane; i < n; i += 32) {
-          float x = up[i], y = uq[i];
-          a = fmaf(x, x, a);
-          b = fmaf(y, y, b);
-          c = fmaf(x, y, c);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          b += __shfl_xor_sync(0xffffffffu, b, o);
-          c += __shfl_xor_sync(0xffffffffu, c, o);
-        }
-        if (fabsf(c) <= tol * sqrtf(a * b)) continue;
-        if (lane == 0) notconv = 1;
-        float zeta = (b - a) / (2.f * c);
-        float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-        float cs = rsqrtf(1.f + t * t), sn = cs * t;
-        for (int i = lane; i < n; i += 32) {
-          float x = up[i], y = uq[i];
-          up[i] = cs * x - sn * y;
-          uq[i] = sn * x + cs * y;
-        }
-      }
-      __syncthreads();
-    }
-    if (!notconv) break;
-    __syncthreads();
+static void jacobi(const LaCtx& la, const double* A, int n, int m, float* gU, float* V, float* W, int max_sweeps,
+                   float tol) {
+  const bool small = n <= kJacobiSmall;
+  const int H = small ? 1 : 4, nb = std::max(2, (ceil_div(n, H) + 1) / 2 * 2);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  cfg.stream = la.stream;
+  if (small) {
+    cfg.gridDim = dim3(1, 1, 1);
+    cfg.blockDim = dim3(32 * nb / 2, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)n * n * sizeof(float);
+    RIHF_CUDA(cudaLaunchKernelEx(&cfg, jacobi1s_kernel<1, 2, 1>, A, n, m, gU, V, W, nb, max_sweeps, tol));
+  } else {
+    cfg.gridDim = dim3(kJacobiCluster, 1, 1);
+    cfg.blockDim = dim3(32 * ceil_div(nb / 2, kJacobiCluster), 1, 1);
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kJacobiCluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    auto run = [&](auto kernel) { RIHF_CUDA(cudaLaunchKernelEx(&cfg, kernel, A, n, m, gU, V, W, nb, max_sweeps, tol)); };
+    if (n <= 128) run(jacobi1s_kernel<4, 4, kJacobiCluster>);
+    else if (n <= 192) run(jacobi1s_kernel<4, 6, kJacobiCluster>);
+    else run(jacobi1s_kernel<4, 8, kJacobiCluster>);
   }
-  jacobi_eigenpairs(U, n, m, sigma, V, W);
-}
-
-// Block one-sided Jacobi (n <= 64 H): the columns form kJB = 64 blocks of H;
-// warp w holds two blocks in registers (H columns x R rows per lane each), and
-// a round rotates every pair across its two blocks (round 0 also the pairs
-// inside each block) before the blocks move on through U in shared memory.
-// The block pairs follow the round-robin order of the column kernel, so a
-// sweep is kJB - 1 rounds instead of n - 1 and moves a third of the shared-
-// memory traffic; column norms are carried as there.
-template <int H>
-__global__ void __launch_bounds__(JT) jacobi1s_block_kernel(const double* __restrict__ A, int n, int m, float* gU,
-                                                            float* V, float* W, int use_smem, int max_sweeps,
-                                                            float tol) {
-  constexpr int R = 2 * H;   // rows per lane
-  extern __shared__ float sm[];
-  __shared__ float red[32];
-  __shared__ float nrm[kJB * H];
-  __shared__ int notconv;
-  float* U = use_smem ? sm : gU;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float sigma = jacobi_shifted_copy(A, n, U, red);
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    if (tid == 0) notconv = 0;
-    for (int j = warp; j < kJB * H; j += JT / 32) {
-      float s2 = 0.f;
-      if (j < n) {
-        const float* u = U + (size_t)j * n;
-        for (int i = lane; i < n; i += 32) s2 = fmaf(u[i], u[i], s2);
-      }
-      for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      if (lane == 0) nrm[j] = s2;
-    }
-    __syncthreads();
-    for (int r = 0; r < kJB - 1; ++r) {
-      int bA, bB;
-      if (warp == 0) {
-        bA = kJB - 1;
-        bB = r;
-      } else {
-        bA = (r + warp) % (kJB - 1);
-        bB = (r - warp + (kJB - 1)) % (kJB - 1);
-      }
-      float x[2 * H][R];
-      float cn[2 * H];
-#pragma unroll
-      for (int c = 0; c < 2 * H; ++c) {
-        const int g = (c < H ? bA * H + c : bB * H + c - H);
-        cn[c] = nrm[g];
-#pragma unroll
-        for (int e = 0; e < R; ++e) {
-          const int i = lane + 32 * e;
-          x[c][e] = (g < n && i < n) ? U[(size_t)g * n + i] : 0.f;
-        }
-      }
-      bool rotated = false;
-      auto rot = [&](float (&xp)[R], float (&xq)[R], float& a, float& b) {
-        float c = 0.f;
-#pragma unroll
-        for (int e = 0; e < R; ++e) c = fmaf(xp[e], xq[e], c);
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (fabsf(c) <= tol * sqrtf(a * b)) return;   // converged pair, or a zero (padding) column
-        rotated = true;
-        const float zeta = (b - a) / (2.f * c);
-        const float t = (zeta >= 0.f ? 1.f : -1.f) / (fabsf(zeta) + sqrtf(1.f + zeta * zeta));
-        const float cs = rsqrtf(1.f + t * t), sn = cs * t;
-#pragma unroll
-        for (int e = 0; e < R; ++e) {
-          const float u = xp[e], v = xq[e];
-          xp[e] = cs * u - sn * v;
-          xq[e] = sn * u + cs * v;
-        }
-        a -= t * c;
-        b += t * c;
-      };
-      if (r == 0) {
-#pragma unroll
-        for (int p = 0; p < H; ++p)
-#pragma unroll
-          for (int q = p + 1; q < H; ++q) {
-            rot(x[p], x[q], cn[p], cn[q]);
-            rot(x[H + p], x[H + q], cn[H + p], cn[H + q]);
-          }
-      }
-#pragma unroll
-      for (int p = 0; p < H; ++p)
-#pragma unroll
-        for (int q = 0; q < H; ++q) rot(x[p], x[H + q], cn[p], cn[H + q]);
-#pragma unroll
-      for (int c = 0; c < 2 * H; ++c) {
-        const int g = (c < H ? bA * H + c : bB * H + c - H);
-        if (g < n) {
-#pragma unroll
-          for (int e = 0; e < R; ++e) {
-            const int i = lane + 32 * e;
-            if (i < n) U[(size_t)g * n + i] = x[c][e];
-          }
-          if (lane == 0) nrm[g] = cn[c];
-        }
-      }
-      if (rotated && lane == 0) notconv = 1;
-      __syncthreads();
-    }
-    if (!notconv) break;
-    __syncthreads();
-  }
-  jacobi_eigenpairs(U, n, m, sigma, V, W);
+  count(la);
 }
 
 // Sort eigenpairs ascending (rank sort) and expand to FP64: X[:, rank] = V[:, i].
@@ -1194,29 +1018,9 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
     dgemm(la, g2);
     Ain = Ag;
   }
-  size_t smem = (size_t)n * n * sizeof(float);
-  int use_smem = smem <= 215 * 1024 ? 1 : 0;
   // a looser stop (n eps) leaves close clusters too coarse for the FP64
   // refinement to separate
-  const float tol = 2e-6f;
-  const int hb = (n + kJB - 1) / kJB;   // block width of the block kernel
-  if (hb <= 3) {
-    const void* fn = hb == 1 ? (const void*)jacobi1s_block_kernel<1>
-                   : hb == 2 ? (const void*)jacobi1s_block_kernel<2> : (const void*)jacobi1s_block_kernel<3>;
-    if (use_smem) raise_smem_limit(fn, (int)smem);
-    const int sz = use_smem ? (int)smem : 0;
-    if (hb == 1)
-      jacobi1s_block_kernel<1><<<1, JT, sz, la.stream>>>(Ain, n, m, fA, fV, fW, use_smem, max_sweeps, tol);
-    else if (hb == 2)
-      jacobi1s_block_kernel<2><<<1, JT, sz, la.stream>>>(Ain, n, m, fA, fV, fW, use_smem, max_sweeps, tol);
-    else
-      jacobi1s_block_kernel<3><<<1, JT, sz, la.stream>>>(Ain, n, m, fA, fV, fW, use_smem, max_sweeps, tol);
-  } else {
-    if (use_smem) raise_smem_limit((const void*)jacobi1s_kernel, (int)smem);
-    jacobi1s_kernel<<<1, JT, use_smem ? smem : 0, la.stream>>>(Ain, n, m, fA, fV, fW, use_smem, max_sweeps, tol);
-  }
-  RIHF_LAUNCH_CHECK();
-  count(la);
+  jacobi(la, Ain, n, m, fA, fV, fW, max_sweeps, 2e-6f);
   eig_sort_kernel<<<std::min(n, 32), 256, 0, la.stream>>>(fV, fW, n, m, V, W);
   RIHF_LAUNCH_CHECK();
   count(la);

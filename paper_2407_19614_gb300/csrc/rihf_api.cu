@@ -1386,12 +1386,13 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
     // refine-only iterations start from them.  Below max|e| = 0.1 (the first
     // iterations after a nuclear step) two sweeps reach ~1e-5 and one
     // refinement and one re-orthonormalisation step suffice; larger errors
-    // (a cold start) take three sweeps and three refinement steps.
+    // (a cold start) take four sweeps and three refinement steps (three sweeps
+    // leave the early iterates, and so the path of DIIS, measurably off).
     const bool light = c->last_err < 0.1;
     graph_or_eager(c, c->diag_graphs[(light ? 4 : 2) + (Fin == c->F ? 0 : 1)], "eigh F' (jacobi+refine)", [&]() {
       form_fp();
       if (light) eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 1, c->Cprev, false, 2, 1);
-      else eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 3, c->Cprev, false, 3);
+      else eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 3, c->Cprev, false, 4);
     });
   } else {
     graph_or_eager(c, c->diag_graphs[Fin == c->F ? 0 : 1], "eigh F' (refine only)", [&]() {
@@ -1437,10 +1438,10 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
     if (!(dev[0] < 1e-8) || !(dev[1] < offd_tol)) {
       if (c->verbose || getenv("RIHF_VERBOSE"))
         fprintf(stderr, "rihf: refine-only eigh deviation %.3e, off-diagonal %.3e, redo\n", dev[0], dev[1]);
-      // warm-started from near-converged vectors: three Jacobi sweeps reach
+      // warm-started from near-converged vectors: four Jacobi sweeps reach
       // the FP32 floor, the four FP64 refinement steps the rest
       TraceScope t(c->tracer, c->stream, "eigh F' (jacobi redo)", 0.0, 0);
-      eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 4, c->Cprev, false, 3);
+      eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 4, c->Cprev, false, 4);
     }
   }
   RIHF_CUDA(cudaMemcpyAsync(c->Cprev, c->Cp, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, c->stream));
