@@ -495,26 +495,84 @@ __global__ void __launch_bounds__(256) trsv_block_kernel(const double* __restric
   }
 }
 
-// Launch shape of trsv_block_kernel: every column is a chain of dependent FP64
-// operations, so narrow blocks spread few columns over many SMs.
-static void trsv_shape(const LaCtx& la, long long ncol, int& blocks, int& threads) {
-  const long long per = (ncol + 2LL * la.sms - 1) / (2LL * la.sms);   // columns per block for two blocks per SM
-  threads = (int)std::min<long long>(256, std::max<long long>(32, (per + 31) / 32 * 32));
-  blocks = (int)std::max<long long>(1, std::min<long long>((ncol + threads - 1) / threads, 16LL * la.sms));
+// The same with eight lanes a column: lane s holds rows s, s + 8, s + 16, s + 24, and
+// each solved entry is passed round by a shuffle.  A column's chain is then about
+// five FP64 instructions an entry instead of up to 32 (10 k clocks instead of 34 k),
+// for 1.6 times the FP64 instructions: faster while the columns leave the SMs short
+// of warps.  The diagonal of l is zero (it is in rd), so rows that are done subtract
+// zero times the entry.
+__global__ void __launch_bounds__(128) trsv_lanes_kernel(const double* __restrict__ L, int n, int k, int b,
+                                                         double* __restrict__ X, long long ncol, int trans) {
+  __shared__ double l[CB][CB + 1];
+  __shared__ double rd[CB];
+  for (int i = threadIdx.x; i < CB * CB; i += 128) {
+    const int r = i / CB, c = i % CB;
+    const double v = r < b && c <= r ? L[(size_t)(k + r) * n + k + c] : 0.0;
+    if (r == c) rd[r] = r < b ? 1.0 / v : 0.0;
+    // trans: the columns of L are walked, so the transpose is kept
+    if (trans) l[c][r] = r == c ? 0.0 : v;
+    else l[r][c] = r == c ? 0.0 : v;
+  }
+  __syncthreads();
+  const int s = threadIdx.x & 7;
+  const long long j = blockIdx.x * 16LL + (threadIdx.x >> 3);
+  double y[CB / 8];
+#pragma unroll
+  for (int q = 0; q < CB / 8; ++q) {
+    const int r = s + 8 * q;
+    y[q] = r < b && j < ncol ? X[(size_t)(k + r) * ncol + j] : 0.0;
+  }
+  if (!trans) {
+#pragma unroll
+    for (int i = 0; i < CB; ++i) {
+      const double v = __shfl_sync(0xffffffffu, y[i / 8] * rd[i], i & 7, 8);
+      if (s == (i & 7)) y[i / 8] = v;
+#pragma unroll
+      for (int q = i / 8; q < CB / 8; ++q) y[q] = fma(-l[s + 8 * q][i], v, y[q]);
+    }
+  } else {
+#pragma unroll
+    for (int i = CB - 1; i >= 0; --i) {
+      const double v = __shfl_sync(0xffffffffu, y[i / 8] * rd[i], i & 7, 8);
+      if (s == (i & 7)) y[i / 8] = v;
+#pragma unroll
+      for (int q = 0; q <= i / 8; ++q) y[q] = fma(-l[s + 8 * q][i], v, y[q]);
+    }
+  }
+  if (j < ncol)
+#pragma unroll
+    for (int q = 0; q < CB / 8; ++q) {
+      const int r = s + 8 * q;
+      if (r < b) X[(size_t)(k + r) * ncol + j] = y[q];
+    }
+}
+
+// One diagonal block of a solve.  Eight lanes a column up to 64 columns an SM (about
+// 9700, where they come to four warps per SM sub-partition: 29 k clocks of FP64
+// instructions against the 34 k of one column's chain in one thread), one thread a
+// column above; narrow blocks then spread few columns over many SMs.
+static void trsv_block(const LaCtx& la, const double* L, int n, int k, int b, double* X, long long ncol, bool trans,
+                       int symcols) {
+  if (ncol <= 64LL * la.sms) {
+    trsv_lanes_kernel<<<(unsigned)((ncol + 15) / 16), 128, 0, la.stream>>>(L, n, k, b, X, ncol, trans ? 1 : 0);
+  } else {
+    const long long per = (ncol + 2LL * la.sms - 1) / (2LL * la.sms);   // columns per block for two blocks per SM
+    const int threads = (int)std::min<long long>(256, std::max<long long>(32, (per + 31) / 32 * 32));
+    const int blocks = (int)std::max<long long>(1, std::min<long long>((ncol + threads - 1) / threads, 16LL * la.sms));
+    trsv_block_kernel<<<blocks, threads, 0, la.stream>>>(L, n, k, b, X, ncol, trans ? 1 : 0, symcols);
+  }
+  RIHF_LAUNCH_CHECK();
+  count(la);
 }
 
 void trsm_lower(const LaCtx& la, const double* L, int n, double* X, long long ncol, bool trans, int symcols,
                 double* tmp) {
   (void)tmp;
   const int nb = ceil_div(n, CB);
-  int blocks, threads;
-  trsv_shape(la, ncol, blocks, threads);
   for (int q = 0; q < nb; ++q) {
     const int kb = trans ? nb - 1 - q : q;
     const int k = kb * CB, b = std::min(CB, n - k);
-    trsv_block_kernel<<<blocks, threads, 0, la.stream>>>(L, n, k, b, X, ncol, trans ? 1 : 0, symcols);
-    RIHF_LAUNCH_CHECK();
-    count(la);
+    trsv_block(la, L, n, k, b, X, ncol, trans, symcols);
     GemmArgs u;
     u.N = (int)ncol; u.K = b;
     u.B = X + (size_t)k * ncol; u.ldb = (int)ncol;
@@ -537,8 +595,6 @@ void trsm_lower(const LaCtx& la, const double* L, int n, double* X, long long nc
 void trsm_lower_tc(const LaCtx& la, const double* L, int n, double* X, long long ncol, int symcols,
                    const TrsmTcScratch& sc) {
   constexpr int PB = kTrsmPanel;   // inner panel width (K of the inner digit-plane updates)
-  int blocks, threads;
-  trsv_shape(la, ncol, blocks, threads);
   // X[r0 + M rows] -= L[r0.., k..k+kk) X[k..k+kk) on the tensor cores
   auto tc_update = [&](int r0, int M, int k, int kk) {
     if (M <= 0) return;
@@ -557,9 +613,7 @@ void trsm_lower_tc(const LaCtx& la, const double* L, int n, double* X, long long
     // the panel in FP64: 32-row substitution blocks and their in-panel updates
     for (int k2 = k; k2 < k + pb; k2 += CB) {
       const int b = std::min(CB, k + pb - k2);
-      trsv_block_kernel<<<blocks, threads, 0, la.stream>>>(L, n, k2, b, X, ncol, 0, symcols);
-      RIHF_LAUNCH_CHECK();
-      count(la);
+      trsv_block(la, L, n, k2, b, X, ncol, false, symcols);
       const int m2 = k + pb - (k2 + b);
       if (m2 > 0) {
         GemmArgs u;
@@ -582,8 +636,6 @@ void trsm_lower_tc(const LaCtx& la, const double* L, int n, double* X, long long
 void trsm_lower_t_tc(const LaCtx& la, const double* L, int n, double* X, long long ncol, int symcols,
                      const TrsmTcScratch& sc) {
   constexpr int PB = kTrsmPanel;
-  int blocks, threads;
-  trsv_shape(la, ncol, blocks, threads);
   // X[r0 .. r0+M) -= L[k..k+kk, r0..r0+M)^T X[k..k+kk) on the tensor cores
   auto tc_update = [&](int r0, int M, int k, int kk) {
     if (M <= 0) return;
@@ -603,9 +655,7 @@ void trsm_lower_t_tc(const LaCtx& la, const double* L, int n, double* X, long lo
       const int kend = std::min(ke, k + PB);
       for (int k2 = k + (kend - k - 1) / CB * CB; k2 >= k; k2 -= CB) {
         const int b = std::min(CB, kend - k2);
-        trsv_block_kernel<<<blocks, threads, 0, la.stream>>>(L, n, k2, b, X, ncol, 1, symcols);
-        RIHF_LAUNCH_CHECK();
-        count(la);
+        trsv_block(la, L, n, k2, b, X, ncol, true, symcols);
         if (k2 > k) {   // rows [k, k2) of the panel: X -= L[k2:k2+b, k:k2]^T X_k2
           GemmArgs u;
           u.M = k2 - k; u.N = (int)ncol; u.K = b;
