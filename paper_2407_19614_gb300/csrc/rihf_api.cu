@@ -208,49 +208,6 @@ void upload(T* d, const std::vector<T>& h, cudaStream_t s) {
 
 // ============================================================ DIIS kernels
 
-// Pulay system [B -1; -1 0] [c; lambda] = [0; -1], B scaled by its largest
-// diagonal entry; Gaussian elimination with partial pivoting (one warp).
-__global__ void diis_solve_kernel(const double* __restrict__ Bm, int ld, int m, double* coef) {
-  __shared__ double a[17][18];
-  int lane = threadIdx.x;
-  int n = m + 1;
-  double sc = 0.0;
-  for (int i = 0; i < m; ++i) sc = fmax(sc, fabs(Bm[i * ld + i]));
-  if (sc == 0.0) sc = 1.0;
-  for (int i = lane; i < n * n; i += 32) {
-    int r = i / n, c = i % n;
-    double v;
-    if (r < m && c < m) v = Bm[r * ld + c] / sc;
-    else if (r == m && c == m) v = 0.0;
-    else v = -1.0;
-    a[r][c] = v;
-  }
-  for (int r = lane; r < n; r += 32) a[r][n] = (r == m) ? -1.0 : 0.0;
-  __syncwarp();
-  for (int k = 0; k < n; ++k) {
-    if (lane == 0) {
-      int piv = k;
-      for (int r = k + 1; r < n; ++r)
-        if (fabs(a[r][k]) > fabs(a[piv][k])) piv = r;
-      if (piv != k)
-        for (int c = 0; c <= n; ++c) {
-          double t = a[k][c];
-          a[k][c] = a[piv][c];
-          a[piv][c] = t;
-        }
-    }
-    __syncwarp();
-    double pk = a[k][k];
-    for (int r = lane; r < n; r += 32) {
-      if (r == k || pk == 0.0) continue;
-      double f = a[r][k] / pk;
-      for (int c = k; c <= n; ++c) a[r][c] -= f * a[k][c];
-    }
-    __syncwarp();
-  }
-  for (int r = lane; r < m; r += 32) coef[r] = a[r][r] != 0.0 ? a[r][n] / a[r][r] : 0.0;
-}
-
 __global__ void diis_extrap_kernel(const double* __restrict__ ring, long long len, int m,
                                    const double* __restrict__ coef, double* out) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x) {
@@ -268,8 +225,8 @@ __global__ void diis_extrap_kernel(const double* __restrict__ ring, long long le
 // leaves a partial in part[], the last block to finish (a ticket counter)
 // folds the partials in block order -- deterministic -- and resets the ticket.
 constexpr int kRedBlocks = 32;
-constexpr int kRedDiis = 8;   // blocks per DIIS dot product
-constexpr int kRedSlots = 128;
+constexpr int kRedDiis = 64;  // blocks of the DIIS dot products (up to 16 vectors)
+constexpr int kRedSlots = 16 * kRedDiis;
 
 __device__ inline double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -357,27 +314,104 @@ __global__ void eig_check_mb_kernel(const double* __restrict__ A, int n, double 
   }
 }
 
-// Row / column s of the DIIS matrix: Bm[s][j] = Bm[j][s] = <e_s, e_j> for j < m,
-// each dot over kRedDiis blocks (blockIdx.x the slice, blockIdx.y = j).
-__global__ void diis_dots_mb_kernel(const double* __restrict__ ring, long long len, int s, int m, double* Bm, int ld,
-                                    double* part, int* ticket) {
-  __shared__ double red[32];
-  const int j = blockIdx.y;
-  const double* a = ring + (long long)s * len;
-  const double* b = ring + (long long)j * len;
-  double v = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x)
-    v += a[i] * b[i];
-  const double t = block_sum(v, red);
-  if (red_finish(t, part, j * kRedDiis + blockIdx.x, ticket) && threadIdx.x == 0) {
-    for (int jj = 0; jj < m; ++jj) {
-      double d = 0.0;
-      for (int k = 0; k < kRedDiis; ++k) d += __ldcg(part + jj * kRedDiis + k);
-      Bm[s * ld + jj] = d;
-      Bm[jj * ld + s] = d;
-    }
-    *ticket = 0;
+// Pulay system [B -1; -1 0] [c; lambda] = [0; -1] of m vectors, B scaled by its
+// largest diagonal entry; Gaussian elimination with partial pivoting by one warp,
+// lane r holding row r (pivots chosen by integer comparison: FP64 comparisons hold
+// the FP64 pipe).
+__device__ inline void diis_solve(const double* Bm, int ld, int m, double* coef) {
+  __shared__ double a[17][18];
+  const int lane = threadIdx.x & 31, n = m + 1;
+  double sc = 0.0;
+  for (int i = 0; i < m; ++i) sc = fmax(sc, fabs(Bm[i * ld + i]));
+  if (sc == 0.0) sc = 1.0;
+  for (int i = lane; i < n * n; i += 32) {
+    const int r = i / n, c = i % n;
+    a[r][c] = r < m && c < m ? Bm[r * ld + c] / sc : (r == m && c == m ? 0.0 : -1.0);
   }
+  for (int r = lane; r < n; r += 32) a[r][n] = r == m ? -1.0 : 0.0;
+  __syncwarp();
+  for (int k = 0; k < n; ++k) {
+    // first row r >= k with the largest |a[r][k]|
+    unsigned long long key = lane >= k && lane < n ? (unsigned long long)__double_as_longlong(fabs(a[lane][k])) : 0ull;
+    int piv = lane >= k && lane < n ? lane : n;
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
+      const int op = __shfl_xor_sync(0xffffffffu, piv, o);
+      if (ok > key || (ok == key && op < piv)) {
+        key = ok;
+        piv = op;
+      }
+    }
+    if (piv != k && piv < n && lane <= n) {   // swap rows k and piv, a column a lane
+      const double t = a[k][lane];
+      a[k][lane] = a[piv][lane];
+      a[piv][lane] = t;
+    }
+    __syncwarp();
+    const double pk = a[k][k];
+    if (lane < n && lane != k && pk != 0.0) {
+      const double f = a[lane][k] / pk;
+      for (int c = k; c <= n; ++c) a[lane][c] -= f * a[k][c];
+    }
+    __syncwarp();
+  }
+  if (lane < m) coef[lane] = a[lane][lane] != 0.0 ? a[lane][n] / a[lane][lane] : 0.0;
+}
+
+// One DIIS step up to the coefficients: F and the error e go into slot s of their
+// rings, row / column s of the DIIS matrix becomes <e, e_j> (j < m), and the block
+// that finishes last solves the Pulay system.  One launch: at the sizes of these
+// vectors the copies, the dot products and the solution were launch latency (33 us
+// an iteration at N = 192 in five launches).
+__global__ void __launch_bounds__(256) diis_push_kernel(const double* __restrict__ F, double* __restrict__ Fring,
+                                                        long long lenF, const double* __restrict__ e,
+                                                        double* __restrict__ Ering, long long len, int s, int m,
+                                                        double* Bm, int ld, double* part, int* ticket, double* coef) {
+  __shared__ double red[8][17];
+  const long long step = (long long)gridDim.x * blockDim.x, first = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (long long i = first; i < lenF; i += step) Fring[(long long)s * lenF + i] = F[i];
+  double v[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = 0.0;
+  for (long long i = first; i < len; i += step) {
+    const double x = e[i];
+    Ering[(long long)s * len + i] = x;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < m) v[j] = fma(x, j == s ? x : Ering[(long long)j * len + i], v[j]);
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    if (j >= m) break;
+    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+    if (lane == 0) red[warp][j] = v[j];
+  }
+  __syncthreads();
+  __shared__ bool last;
+  if (threadIdx.x < m) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    part[threadIdx.x * gridDim.x + blockIdx.x] = t;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int j = warp; j < m; j += 8) {   // a warp per vector, the partial sums in a fixed order
+    double t = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + j * gridDim.x + b);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+      Bm[s * ld + j] = t;
+      Bm[j * ld + s] = t;
+    }
+  }
+  if (threadIdx.x == 0) *ticket = 0;
+  __syncthreads();
+  if (warp == 0 && m >= 2) diis_solve(Bm, ld, m, coef);
 }
 
 // ============================================================ tracing
@@ -2352,9 +2386,6 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     cudaEventRecord(c->ev[3], s);
     int slot = (it - 1 - dbase) % size;
     int m = std::min(it - dbase, size);
-    RIHF_CUDA(cudaMemcpyAsync(c->Fring + slot * n2, c->F, sizeof(double) * n2, cudaMemcpyDeviceToDevice, s));
-    RIHF_CUDA(cudaMemcpyAsync(c->Ering + (size_t)slot * n * n, c->Err, sizeof(double) * n * n,
-                              cudaMemcpyDeviceToDevice, s));
     double sc[2];
     RIHF_CUDA(cudaMemcpyAsync(sc, c->scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaStreamSynchronize(s));
@@ -2405,18 +2436,18 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     const double* Fuse = c->F;
     if (!restart) {
       TraceScope t(c->tracer, s, "DIIS (dots, solve, extrapolation)", 0.0, 0);
-      diis_dots_mb_kernel<<<dim3(kRedDiis, m), 256, 0, s>>>(c->Ering, (long long)n * n, slot, m, c->Bdiis, 16, c->d_red,
-                                                             c->d_ticket);
+      diis_push_kernel<<<(int)std::min<long long>(kRedDiis, std::max<long long>(1, ((long long)n2 + 255) / 256)), 256, 0, s>>>(
+          c->F, c->Fring, (long long)n2, c->Err, c->Ering, (long long)n * n, slot, m, c->Bdiis, 16, c->d_red, c->d_ticket,
+          c->coef);
       RIHF_LAUNCH_CHECK();
       if (m >= 2) {
-        diis_solve_kernel<<<1, 32, 0, s>>>(c->Bdiis, 16, m, c->coef);
         diis_extrap_kernel<<<std::max(1, std::min(ceil_div((long long)n2, 256), 8 * c->sms)), 256, 0, s>>>(
             c->Fring, (long long)n2, m, c->coef, c->Fx);
         RIHF_LAUNCH_CHECK();
         Fuse = c->Fx;
       }
     }
-    if (!restart) c->launches += 3;
+    if (!restart) c->launches += 2;
     // no host synchronisation here: the next Fock build queues behind the
     // diagonalisation on the stream
     diagonalise(c, Fuse, true);
