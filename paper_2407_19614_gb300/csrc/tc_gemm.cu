@@ -2,6 +2,7 @@
 // operands staged in shared memory by bulk asynchronous copies.  See
 // tc_gemm.cuh for the number format.
 #include <algorithm>
+#include <cmath>
 
 #include "../../include/rihf.h"
 #include "tc_gemm.cuh"
@@ -80,20 +81,27 @@ __device__ inline void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// D (TMEM) = A (smem) . B (smem)^T [+ D], BF16 inputs, FP32 accumulator.
-__device__ inline void mma_bf16(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+// D (TMEM) = A (smem) . B (smem)^T [+ D], BF16 inputs, FP32 accumulator; issued by
+// the one lane of the warp with lead != 0 (a predicate, so that the warp stays
+// converged and the operands stay in uniform registers).
+__device__ inline void mma_bf16(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc,
+                                uint32_t lead) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(lead)
       : "memory");
 }
 
-__device__ inline void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_addr(bar))
-               : "memory");
+__device__ inline void mma_commit(uint64_t* bar, uint32_t lead) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_addr(bar)),
+      "r"(lead)
+      : "memory");
 }
 
 // 32 lanes x 8 consecutive 32-bit columns; thread i gets lane (base + i).
@@ -105,6 +113,20 @@ __device__ inline void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 }
 
 __device__ inline void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// One 32-byte sector of a row (p 32-byte aligned).
+__device__ inline void ld_sector(const double* p, double* v) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+               : "l"(__cvta_generic_to_global(p))
+               : "memory");
+}
+
+__device__ inline void st_sector(double* p, const double* v) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "d"(v[0]), "d"(v[1]),
+               "d"(v[2]), "d"(v[3])
+               : "memory");
+}
 
 // Shared-memory matrix descriptor, no swizzle, K-major core matrices of
 // 8 rows x 16 bytes: 128 B between K-adjacent core matrices (leading byte
@@ -138,25 +160,23 @@ __device__ inline uint32_t bf16_of_int(int d) {
   return __float_as_uint(f) >> 16;
 }
 
-// S * 2^e2 as the nearest double (integer construction, no FP64 arithmetic).
+// S * 2^e2 as the nearest double (ties to even), 0 below the normal range: integer
+// construction, no FP64 arithmetic and no branches, so that the conversions of
+// a thread's elements overlap.
 __device__ inline double oz_to_double(long long S, int e2) {
-  if (S == 0) return 0.0;
-  const unsigned long long sign = S < 0 ? (1ULL << 63) : 0ULL;
-  const unsigned long long a = S < 0 ? (unsigned long long)(-S) : (unsigned long long)S;
-  const int lz = __clzll((long long)a);
-  const unsigned long long n = a << lz;
-  unsigned long long m = n >> 11;
-  const unsigned long long rem = n & 0x7FF;
-  if (rem > 0x400 || (rem == 0x400 && (m & 1))) ++m;
-  int ex = 63 - lz + e2;
-  if (m >> 53) {
-    m >>= 1;
-    ++ex;
-  }
-  const int be = ex + 1023;
-  if (be <= 0) return 0.0;
-  if (be >= 2047) return __longlong_as_double((long long)(sign | (0x7FFULL << 52)));
-  return __longlong_as_double((long long)(sign | ((unsigned long long)be << 52) | (m & ((1ULL << 52) - 1))));
+  const unsigned long long a = (unsigned long long)(S < 0 ? -S : S);
+  const int lz = __clzll((long long)a);                     // 64 when S = 0
+  const unsigned long long n = a << (lz & 63);
+  // mantissa with its leading bit (53 bits), rounded; a carry out of it moves
+  // into the exponent field by the addition below
+  const unsigned long long m = (n >> 11) + ((n & 0x7FF) + ((n >> 11) & 1) > 0x400 ? 1ULL : 0ULL);
+  const int be = 63 - lz + e2 + 1023;                        // biased exponent before a carry
+  unsigned long long bits = ((unsigned long long)(uint32_t)(be - 1) << 52) + m;
+  const int bc = be + (int)(m >> 53);
+  if (bc <= 0 || S == 0) bits = 0ULL;
+  if (bc >= 2047 && S != 0) bits = 0x7FFULL << 52;
+  if (S < 0 && bc > 0) bits |= 1ULL << 63;
+  return __longlong_as_double((long long)bits);
 }
 
 // ------------------------------------------------------------ slicing
@@ -250,12 +270,21 @@ __global__ void __launch_bounds__(kOzThreads) oz_slice_kernel(OzSrc S, int kchun
 // the SMs stay balanced.
 //   warp 9 (one lane): takes items, streams their K chunks' digit planes into
 //     a ring of shared-memory stages with bulk copies;
-//   warp 8 (one lane): issues the MMAs of each chunk, diagonal by diagonal, and
-//     commits stage releases and, every G chunks, a full accumulator group;
+//   warp 8: issues the MMAs of each chunk and commits stage releases and, every
+//     G chunks, a full accumulator group;
 //   warps 0-7: drain the s TMEM accumulators of each group (a row and half the
-//     columns per thread) into int64 fixed-point sums; each diagonal is
-//     released (its own mbarrier) as soon as it is in registers, so the next
-//     group's MMAs on it overlap the conversion of the rest.
+//     columns per thread) into int64 fixed-point sums; the group is released when
+//     its last columns are in registers, so the next group's MMAs overlap the
+//     rest of the conversion and, at a tile's end, the stores.
+// The kernel is compiled per digit count and column tile: every descriptor offset
+// and diagonal weight is then a constant.  With run-time counts one MMA took 138
+// clocks to issue (its table entry, its operands' way into uniform registers)
+// against the 90 it runs, a tile's diagonals 4.8 k clocks to read (now 2.4 k) and
+// its epilogue 20 k (now 12 k: no FP64 product for alpha = +-2^n, exponents
+// fetched ahead, 32-byte stores); 77824 x 64, K = 384, 7 digits: 303 -> 212 k
+// clocks a CTA, the tensor pipe active 30 -> 41 %.  What remains is the read-out
+// between groups, which the 512 TMEM columns leave no room to overlap, and for
+// operands from HBM the two stages that shared memory holds.
 // A group spans G = floor(1024 / s) / kOzChunk chunks: every diagonal sum then
 // stays below s * 32G * 128^2 <= 2^24 and is exact in FP32.  Every wait is
 // bounded; the first one that runs out raises a shared abort flag, all roles
@@ -271,15 +300,9 @@ constexpr int kSmemMax = 227 * 1024;
 constexpr int kSmemMin = 116 * 1024;   // more than half an SM's shared memory: one CTA per SM
 constexpr int kBookBytes = 1024;
 
-// One MMA of a K chunk, precomputed: TMEM column offset (bit 31: the MMA
-// starts its accumulator when the chunk opens a group), A and B descriptor
-// address offsets in 16-byte units, instruction descriptor.
-constexpr int kMaxChunkMmas = 32;
-
 struct OzBook {
-  uint4 mmas[kMaxChunkMmas];
   uint64_t full[kMaxStages], empty[kMaxStages];
-  uint64_t accfull, accempty[kOzMaxDigits];
+  uint64_t accfull, accempty;
   uint64_t item_full[kItemSlots], item_empty[kItemSlots];
   int item[kItemSlots];
   uint32_t tslot;
@@ -293,6 +316,7 @@ struct OzTiling {
   int M, N, TN, mtiles, ntiles, nsplit, nitems, nfast;
   int lower_only, symcols, kb_chunks, kchunks;
   int s, G, nst, stage_bytes;
+  int aexp, aneg, scale;   // alpha = +-2^aexp (scale 0), or it is multiplied
 };
 
 __device__ inline void mbar_arrive(uint64_t* bar) {
@@ -344,6 +368,17 @@ __device__ inline bool oz_valid(const OzTiling& T, int mt, int nt, int c0, int c
   return true;
 }
 
+// The integer in accumulator d (d + 1 digit pairs of at most 2^14 K'(S) each): by an
+// FP32 addition where that stays within 2^22, else by a conversion instruction,
+// which only the slow unit has (16 a clock and SM: the read-out is bound by it).
+template <int S>
+__device__ inline int oz_sum_to_int(int d, float x) {
+  constexpr int kp = (1024 / S) / kOzChunk * kOzChunk;   // elements accumulated between read-outs
+  if ((d + 1) * kp <= 256) return __float_as_int(x + 12582912.0f) - 0x4B400000;
+  return __float2int_rn(x);
+}
+
+template <int S, int TN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     oz_gemm_kernel(OzOperand A, OzOperand B, OzTiling T, double alpha, double* C, long long MR, long long cs_m1,
                    long long cs_m2, long long cs_n, int atomic, int* flag, int* sched) {
@@ -351,9 +386,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   OzBook* bk = reinterpret_cast<OzBook*>(smem + (size_t)T.nst * T.stage_bytes);
   volatile int* abort = &bk->abort;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int s = T.s, TN = T.TN;
-  const uint32_t a_bytes = (uint32_t)s * kPlaneElems * 2, b_plane = (uint32_t)TN * kOzChunk * 2;
+  // the warp index by a shuffle: the roles' branches are then known to be uniform
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  constexpr uint32_t s = S, a_bytes = s * kPlaneElems * 2, b_plane = TN * kOzChunk * 2;
 
   if (tid == 0) {
     for (int i = 0; i < T.nst; ++i) {
@@ -362,7 +397,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
     mbar_init(&bk->accfull, 1);
     // one arrival per drain warp (its lane 0, after the warp's reads)
-    for (int d = 0; d < kOzMaxDigits; ++d) mbar_init(&bk->accempty[d], kDrainThreads / 32);
+    mbar_init(&bk->accempty, kDrainThreads / 32);
     for (int k = 0; k < kItemSlots; ++k) {
       mbar_init(&bk->item_full[k], 1);
       mbar_init(&bk->item_empty[k], kDrainThreads / 32 + 1);
@@ -405,7 +440,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           uint8_t* Bs = As + a_bytes;
           mbar_expect_tx(&bk->full[st], a_bytes + (uint32_t)s * b_plane);
           bulk_load(As, A.planes + ((size_t)mt * A.kchunks + c) * A.smax * kPlaneElems, a_bytes, &bk->full[st]);
-          for (int u = 0; u < s; ++u)
+          for (uint32_t u = 0; u < s; ++u)
             bulk_load(Bs + u * b_plane,
                       B.planes + (((size_t)b_rt * B.kchunks + c) * B.smax + u) * kPlaneElems +
                           (size_t)b_off * kOzChunk,
@@ -423,88 +458,83 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
     __syncwarp();
   } else if (warp == 8) {
-    if (lane == 0) {   // ---------------- MMA issuer
-      // BF16 x BF16 -> FP32, M = 128; N is set per MMA
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kOzTileM >> 4) << 24);
-      const int planes_per_mma = 256 / TN;
-      // the MMAs of one chunk: per K step j, A plane t and group of B planes,
-      // one MMA; the B planes u = 1..s+1-t lie one after another in shared
-      // memory with the same 8-row-group stride, so up to 256 / TN of them form
-      // one operand of N = count * TN rows, and the product (t, u) lands on the
-      // columns of anti-diagonal t + u.  Built once: the issue loop then costs
-      // a table load and two adds per MMA instead of the index arithmetic.
-      int nm = 0;
-      for (int j = 0; j < kOzChunk / 16; ++j)
-        for (int t = 1; t <= s; ++t)
-          for (int u0 = 1; u0 <= s + 1 - t; u0 += planes_per_mma) {
-            const int np = min(planes_per_mma, s + 2 - t - u0);
-            uint4 m;
-            m.x = (uint32_t)((t + u0 - 2) * TN) | ((t == 1 && j == 0) ? 0x80000000u : 0u);
-            m.y = (uint32_t)(((t - 1) * kPlaneElems * 2 + j * 256) >> 4);
-            m.z = (uint32_t)(((u0 - 1) * b_plane + j * 256) >> 4);
-            m.w = idesc0 | ((uint32_t)((np * TN) >> 3) << 17);
-            if (nm < kMaxChunkMmas) bk->mmas[nm] = m;
-            ++nm;
-          }
-      if (nm > kMaxChunkMmas) {   // cannot happen for s <= 7 and TN >= 16 (at most 28)
-        *abort = 1;
-        nm = 0;
-      }
-      uint32_t i = 0, grp = 0;
-      int last_st = -1;
-      uint32_t last_par = 0;
-      bool ok = !*abort;
-      for (int q = 0; ok; ++q) {
-        const int slot = q % kItemSlots;
-        if (!oz_wait(&bk->item_full[slot], (q / kItemSlots) & 1, abort)) break;
-        const int idx = *(volatile int*)&bk->item[slot];
-        mbar_arrive(&bk->item_empty[slot]);
-        if (idx < 0) break;
-        int mt, nt, split, c0, c1;
-        oz_decode(T, idx, mt, nt, split, c0, c1);
-        for (int c = c0; c < c1; ++c, ++i) {
-          const int st = (int)(i % (uint32_t)T.nst);
-          if (!oz_wait(&bk->full[st], (i / T.nst) & 1, abort)) {
+    // ---------------- MMA issuer: the warp stays converged, lane 0 issues
+    // BF16 x BF16 -> FP32, M = 128; N is set per MMA
+    const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kOzTileM >> 4) << 24);
+    constexpr int planes_per_mma = 256 / TN;
+    const uint32_t lead = lane == 0 ? 1u : 0u;
+    // a wait whose result the lanes agree on
+    auto wait_all = [&](uint64_t* bar, uint32_t parity) -> bool {
+      return __all_sync(0xffffffffu, oz_wait(bar, parity, abort));
+    };
+    uint32_t i = 0, grp = 0;
+    int last_st = -1;
+    uint32_t last_par = 0;
+    bool ok = true;
+    for (int q = 0; ok; ++q) {
+      const int slot = q % kItemSlots;
+      if (!wait_all(&bk->item_full[slot], (q / kItemSlots) & 1)) break;
+      const int idx = __shfl_sync(0xffffffffu, *(volatile int*)&bk->item[slot], 0);
+      if (lane == 0) mbar_arrive(&bk->item_empty[slot]);
+      if (idx < 0) break;
+      int mt, nt, split, c0, c1;
+      oz_decode(T, idx, mt, nt, split, c0, c1);
+      for (int c = c0; c < c1; ++c, ++i) {
+        const int st = (int)(i % (uint32_t)T.nst);
+        if (!wait_all(&bk->full[st], (i / T.nst) & 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const bool first = (c - c0) % T.G == 0, last = (c - c0) % T.G == T.G - 1 || c == c1 - 1;
+        if (first && grp > 0) {   // the last group read out
+          if (!wait_all(&bk->accempty, (grp - 1) & 1)) {
             ok = false;
+            ++i;
             break;
           }
           tc_fence_after();
-          const bool first = (c - c0) % T.G == 0, last = (c - c0) % T.G == T.G - 1 || c == c1 - 1;
-          if (first && grp > 0) {   // every diagonal of the last group read out
-            for (int d = 0; d < s && ok; ++d)
-              if (!oz_wait(&bk->accempty[d], (grp - 1) & 1, abort)) ok = false;
-            if (!ok) {
-              ++i;
-              break;
+        }
+        // per K step j, A plane t and group of B planes, one MMA; the B planes
+        // u = 1..s+1-t lie one after another in shared memory with the same
+        // 8-row-group stride, so up to 256 / TN of them form one operand of
+        // N = count * TN rows, and the product (t, u) lands on the columns of
+        // anti-diagonal t + u.  Plane and K-step offsets go into the 14-bit
+        // address field of the stage's descriptors (shared addresses stay
+        // below 256 KB).
+        const uint32_t a_s = smem_addr(smem + (size_t)st * T.stage_bytes);
+        const uint64_t a_d0 = smem_desc(a_s), b_d0 = smem_desc(a_s + a_bytes);
+#pragma unroll
+        for (int j = 0; j < kOzChunk / 16; ++j) {
+#pragma unroll
+          for (int t = 0; t < S; ++t) {
+            const uint64_t a_d = a_d0 + (uint64_t)((t * kPlaneElems * 2 + j * 256) >> 4);
+            const uint32_t acc = t == 0 && j == 0 && first ? 0u : 1u;
+#pragma unroll
+            for (int u = 0; u < S - t; u += planes_per_mma) {
+              constexpr int most = planes_per_mma;
+              const int np = most < S - t - u ? most : S - t - u;
+              mma_bf16(taddr + (uint32_t)((t + u) * TN), a_d, b_d0 + (uint64_t)((u * (int)b_plane + j * 256) >> 4),
+                       idesc0 | ((uint32_t)((np * TN) >> 3) << 17), acc, lead);
             }
-            tc_fence_after();
-          }
-          // descriptors of the stage's first planes; plane and K-step offsets go
-          // into the 14-bit address field (shared addresses stay below 256 KB)
-          const uint32_t a_s = smem_addr(smem + (size_t)st * T.stage_bytes);
-          const uint64_t a_d0 = smem_desc(a_s), b_d0 = smem_desc(a_s + a_bytes);
-#pragma unroll 4
-          for (int e = 0; e < nm; ++e) {
-            const uint4 m = bk->mmas[e];
-            const uint32_t init = (m.x >> 31) & (first ? 1u : 0u);
-            mma_bf16(taddr + (m.x & 0x7FFFFFFFu), a_d0 + m.y, b_d0 + m.z, m.w, init ^ 1u);
-          }
-          mma_commit(&bk->empty[st]);   // the stage is free once these MMAs are done
-          last_st = st;
-          last_par = (i / T.nst) & 1;
-          if (last) {
-            mma_commit(&bk->accfull);
-            ++grp;
           }
         }
+        mma_commit(&bk->empty[st], lead);   // the stage is free once these MMAs are done
+        last_st = st;
+        last_par = (i / T.nst) & 1;
+        if (last) {
+          mma_commit(&bk->accfull, lead);
+          ++grp;
+        }
       }
-      bk->consumed = (int)i;
-      if (*abort && last_st >= 0) mbar_wait(&bk->empty[last_st], last_par);   // MMAs in flight
     }
+    if (lane == 0) bk->consumed = (int)i;
+    if (*abort && last_st >= 0) mbar_wait(&bk->empty[last_st], last_par);   // MMAs in flight
     __syncwarp();
   } else {   // ---------------- drain: warps 0-7
     const int row = 32 * (warp & 3) + lane;
-    const int ncol = TN / 2, col0 = (warp >> 2) * ncol;
+    constexpr int ncol = TN / 2;
+    const int col0 = (warp >> 2) * ncol;
     const uint32_t t_row = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
     // one thread polls, the other drain threads wait on a hardware named
     // barrier (spinning 256 threads would compete with the copy and MMA
@@ -529,84 +559,105 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       if (idx < 0) break;
       int mt, nt, split, c0, c1;
       oz_decode(T, idx, mt, nt, split, c0, c1);
-      long long acc[kOzMaxTN / 2];
+      // the exponents (padded to whole tiles) are fetched ahead of their use:
+      // lane k's eb is that of column k of the warp's ncol <= 32
+      const int m = mt * kOzTileM + row, n0 = nt * TN + col0;
+      const int ea = A.exps[(size_t)m * A.nkb + split] - 2095 + T.aexp;
+      const int eb = lane < ncol ? B.exps[(size_t)(n0 + lane) * B.nkb + split] : 0;
+      long long acc[ncol];
 #pragma unroll
-      for (int k = 0; k < kOzMaxTN / 2; ++k) acc[k] = 0;
+      for (int k = 0; k < ncol; ++k) acc[k] = 0;
       for (int c = c0; c < c1 && ok; c += T.G) {
         ok = drain_wait(&bk->accfull, grp & 1);
         if (!ok) break;
         tc_fence_after();
-        for (int g = 2; g <= s + 1; ++g) {
-          const int sh = 37 - 8 * (g - 2);
-          const uint32_t tg = t_row + (uint32_t)((g - 2) * TN + col0);
-          uint32_t r[kOzMaxTN / 16][8];
+        // eight columns of all s diagonals at a time (the warp's last block read
+        // frees the accumulators): the element's sum then has constant weights
+        // 2^37, 2^29, ... 2^-11, one multiply-add each
 #pragma unroll
-          for (int q8 = 0; q8 < kOzMaxTN / 16; ++q8)
-            if (8 * q8 < ncol) tmem_ld8(tg + 8 * q8, r[q8]);
+        for (int q8 = 0; q8 < ncol / 8; ++q8) {
+          uint32_t r[S][8];
+#pragma unroll
+          for (int d = 0; d < S; ++d) tmem_ld8(t_row + (uint32_t)(d * TN + col0 + 8 * q8), r[d]);
           tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&bk->accempty[g - 2]);
+          if (q8 == ncol / 8 - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bk->accempty);
+          }
 #pragma unroll
-          for (int q8 = 0; q8 < kOzMaxTN / 16; ++q8) {
-            if (8 * q8 < ncol) {
+          for (int e = 0; e < 8; ++e) {
+            long long a = acc[8 * q8 + e];
+            int low = 0;
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                const long long v = (long long)__float2int_rn(__uint_as_float(r[q8][e]));
-                acc[8 * q8 + e] += sh >= 0 ? (v << sh) : (v >> (-sh));
-              }
+            for (int d = 0; d < S; ++d) {
+              const int v = oz_sum_to_int<S>(d, __uint_as_float(r[d][e]));
+              const int sh = 37 - 8 * d;
+              if (sh >= 0) a += (long long)v * (1LL << (sh < 0 ? 0 : sh));
+              else low += v >> (sh < 0 ? -sh : 0);
             }
+            if (S > 5) a += low;
+            acc[8 * q8 + e] = a;
           }
         }
         ++grp;
       }
       if (!ok) break;
-      const long long m = (long long)mt * kOzTileM + row;
-      if (m < T.M) {
-        // all of the thread's values first (the exponent loads overlap), then
-        // the stores: 16-byte pairs when the row is contiguous and aligned
-        const int ea = A.exps[(size_t)m * A.nkb + split] - 2095;
-        const int n0 = nt * TN + col0;
-        const int nv = min(ncol, T.N - n0);
-        double v[kOzMaxTN / 2];
+      // all of the thread's values first, then the stores: whole 32-byte sectors
+      // when the row is contiguous and aligned (16-byte halves write a sector twice)
+      const int nv = min(ncol, T.N - n0);
+      double v[ncol];
 #pragma unroll
-        for (int k = 0; k < kOzMaxTN / 2; ++k) {
-          v[k] = 0.0;
-          if (k < nv) {
-            v[k] = oz_to_double(acc[k], ea + B.exps[(size_t)(n0 + k) * B.nkb + split]);
-            if (alpha != 1.0) v[k] *= alpha;
-          }
-        }
-        double* dst = C + (m % MR) * cs_m1 + (m / MR) * cs_m2 + (long long)n0 * cs_n;
+      for (int k = 0; k < ncol; ++k) {
+        v[k] = oz_to_double(T.aneg ? -acc[k] : acc[k], ea + __shfl_sync(0xffffffffu, eb, k));
+      }
+      if (T.scale)   // not a predicate on each product: those hold the FP64 pipe also when it is false
+#pragma unroll
+        for (int k = 0; k < ncol; ++k) v[k] *= alpha;
+      const int mr = MR < T.M ? (int)MR : T.M;
+      double* dst = C + (long long)(m % mr) * cs_m1 + (long long)(m / mr) * cs_m2 + (long long)n0 * cs_n;
+      const bool sectors =
+          __all_sync(0xffffffffu, m >= T.M || (cs_n == 1 && nv == ncol && ((uintptr_t)dst & 31) == 0));
+      if (m < T.M) {
         if (atomic == 1) {
 #pragma unroll
-          for (int k = 0; k < kOzMaxTN / 2; ++k)
+          for (int k = 0; k < ncol; ++k)
             if (k < nv) atomicAdd(dst + (long long)k * cs_n, v[k]);
+        } else if (sectors) {
+#pragma unroll
+          for (int k0 = 0; k0 < ncol; k0 += 8) {   // two sectors in flight at a time
+            if (atomic == 2) {
+              double old[8];
+              ld_sector(dst + k0, old);
+              ld_sector(dst + k0 + 4, old + 4);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) v[k0 + k] = old[k] + v[k0 + k];
+            }
+            st_sector(dst + k0, v + k0);
+            st_sector(dst + k0 + 4, v + k0 + 4);
+          }
         } else if (cs_n == 1 && ((uintptr_t)dst & 15) == 0) {
           double2* d2 = reinterpret_cast<double2*>(dst);
-          if (atomic == 2) {
 #pragma unroll
-            for (int k0 = 0; k0 < kOzMaxTN / 4; k0 += 4) {   // four pairs in flight at a time
-              double2 old[4];
+          for (int k0 = 0; k0 < ncol / 2; k0 += 4) {   // four pairs in flight at a time
+            double2 old[4];
 #pragma unroll
-              for (int k = k0; k < k0 + 4; ++k)
-                if (2 * k + 1 < nv) old[k - k0] = d2[k];
+            for (int k = k0; k < k0 + 4; ++k)
+              old[k - k0] = atomic == 2 && 2 * k + 1 < nv ? d2[k] : make_double2(0.0, 0.0);
 #pragma unroll
-              for (int k = k0; k < k0 + 4; ++k) {
-                if (2 * k + 1 < nv) d2[k] = make_double2(old[k - k0].x + v[2 * k], old[k - k0].y + v[2 * k + 1]);
-                else if (2 * k < nv) dst[2 * k] += v[2 * k];
+            for (int k = k0; k < k0 + 4; ++k) {
+              if (2 * k + 1 < nv) {
+                if (atomic == 2) d2[k] = make_double2(old[k - k0].x + v[2 * k], old[k - k0].y + v[2 * k + 1]);
+                else d2[k] = make_double2(v[2 * k], v[2 * k + 1]);
+              } else if (2 * k < nv) {
+                if (atomic == 2) dst[2 * k] += v[2 * k];
+                else dst[2 * k] = v[2 * k];
               }
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < kOzMaxTN / 4; ++k) {
-              if (2 * k + 1 < nv) d2[k] = make_double2(v[2 * k], v[2 * k + 1]);
-              else if (2 * k < nv) dst[2 * k] = v[2 * k];
             }
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < kOzMaxTN / 2; ++k) {
+          for (int k = 0; k < ncol; ++k) {
             if (k < nv) {
               double* d = dst + (long long)k * cs_n;
               if (atomic == 2) *d += v[k];
@@ -631,6 +682,27 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   if (warp == 8) {
     tc_fence_after();
     tmem_dealloc(taddr, kTmemCols);
+  }
+}
+
+using OzKernel = void (*)(OzOperand, OzOperand, OzTiling, double, double*, long long, long long, long long, long long,
+                          int, int*, int*);
+
+template <int S>
+OzKernel oz_kernel_tn(int tn) {
+  return tn <= 16 ? oz_gemm_kernel<S, 16> : tn <= 32 ? oz_gemm_kernel<S, 32> : tn <= 48 ? oz_gemm_kernel<S, 48>
+                                                                                   : oz_gemm_kernel<S, 64>;
+}
+
+OzKernel oz_kernel(int s, int tn) {
+  switch (s) {
+    case 1: return oz_kernel_tn<1>(tn);
+    case 2: return oz_kernel_tn<2>(tn);
+    case 3: return oz_kernel_tn<3>(tn);
+    case 4: return oz_kernel_tn<4>(tn);
+    case 5: return oz_kernel_tn<5>(tn);
+    case 6: return oz_kernel_tn<6>(tn);
+    default: return oz_kernel_tn<7>(tn);
   }
 }
 
@@ -694,6 +766,26 @@ OzOperand oz_slice(const LaCtx& la, const double* X, int rows, int K, long long 
   return op;
 }
 
+// Column tile of a GEMM that does not state one.  A tile's time grows with its
+// columns, so while narrow tiles leave SMs idle they cost nothing: the narrowest
+// of 16, 32 with at most one tile an SM (n = 384, 7 digits: 28 / 33 / 55 k clocks at
+// 16 / 32 / 64; n = 192: 18 / 23 / 39 k).  Above that the operand loads of a tile
+// are what repeats, and the widest is best (1024 x 12000, K = 256: 596 / 352 / 330 k),
+// with 65..96 columns as two tiles of 48 (80 columns: 267 / 327 k at 48 / 64 and
+// 7 digits, 176 / 200 k at 5).  No tile straddles a 128-row plane: the widths divide
+// 128 or all tiles lie in the first one.
+static int oz_column_tile(int M, int N, int nsplit, bool lower_only, int sms) {
+  const long long rows = (long long)(M + kOzTileM - 1) / kOzTileM * nsplit;
+  for (int tn : {16, 32}) {
+    if (N <= tn) return tn;
+    long long tiles = rows * ((N + tn - 1) / tn);
+    if (lower_only) tiles = tiles / 2 + rows * (kOzTileM / tn) / 2;   // those on and below the diagonal
+    if (tiles <= sms) return tn;
+  }
+  if (N <= kOzMaxTN) return (N + 15) / 16 * 16;
+  return N <= 96 ? 48 : kOzMaxTN;
+}
+
 void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   if (g.M <= 0 || g.N <= 0) return;
   const OzOperand &A = g.A, &B = g.B;
@@ -705,14 +797,14 @@ void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   if (!g.atomic && A.nkb > 1) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: K blocks need atomic output");
   if (g.atomic && g.accumulate) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: atomic and accumulate");
   if (!la.sched) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: no work counter");
-  // column tile: the whole of N when it fits (multiple of 16), else kOzMaxTN
-  // (a divisor of 128, so no tile straddles a 128-row plane)
   OzTiling T;
   T.M = g.M;
   T.N = g.N;
-  if (g.tn < 0 || g.tn % 16 || g.tn > kOzMaxTN || (g.tn > 0 && g.N > g.tn && 128 % g.tn))
+  if (g.tn < 0 || g.tn % 16 || g.tn > kOzMaxTN ||
+      (g.tn > 0 && g.N > g.tn && 128 % g.tn && (g.N + g.tn - 1) / g.tn * g.tn > 128))
     throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: bad column tile");
-  T.TN = g.tn > 0 ? g.tn : (g.N <= kOzMaxTN ? (g.N + 15) / 16 * 16 : kOzMaxTN);
+  const int sms = la.sms > 0 ? la.sms : 152;
+  T.TN = g.tn > 0 ? g.tn : oz_column_tile(g.M, g.N, A.nkb, g.lower_only, sms);
   T.s = g.s;
   if (T.s * T.TN > kTmemCols) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: accumulators exceed TMEM");
   T.mtiles = (g.M + kOzTileM - 1) / kOzTileM;
@@ -730,10 +822,18 @@ void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   T.stage_bytes = T.s * (kPlaneElems * 2 + T.TN * kOzChunk * 2);
   T.nst = std::min(kMaxStages, (kSmemMax - kBookBytes - 1024) / T.stage_bytes);
   if (T.nst < 1) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: stage exceeds shared memory");
+  // a power of two goes into the integer result instead of an FP64 product
+  int aexp = 0;
+  const double amant = std::frexp(g.alpha, &aexp);
+  const bool pow2 = std::fabs(amant) == 0.5;
+  T.aexp = pow2 ? aexp - 1 : 0;
+  T.aneg = pow2 && g.alpha < 0.0 ? 1 : 0;
+  T.scale = pow2 ? 0 : 1;
   const int smem = std::max(kSmemMin, T.nst * T.stage_bytes + kBookBytes + 1024);
-  raise_smem_limit((const void*)oz_gemm_kernel, kSmemMax);
-  const int grid = (int)std::min<long long>(nitems, la.sms > 0 ? la.sms : 152);
-  oz_gemm_kernel<<<grid, kGemmThreads, smem, la.stream>>>(A, B, T, g.alpha, g.C, g.MR, g.cs_m1, g.cs_m2, g.cs_n,
+  const OzKernel kernel = oz_kernel(T.s, T.TN);
+  raise_smem_limit((const void*)kernel, kSmemMax);
+  const int grid = (int)std::min<long long>(nitems, sms);
+  kernel<<<grid, kGemmThreads, smem, la.stream>>>(A, B, T, g.alpha, g.C, g.MR, g.cs_m1, g.cs_m2, g.cs_n,
                                                           g.atomic ? 1 : (g.accumulate ? 2 : 0), la.flag, la.sched);
   RIHF_LAUNCH_CHECK();
   if (la.launches) *la.launches += 1;
