@@ -154,12 +154,6 @@ __device__ inline long long oz_fixed(double x, int E) {
   return (bits >> 63) ? -V : V;
 }
 
-// BF16 bit pattern of a small integer |d| <= 256 (exact).
-__device__ inline uint32_t bf16_of_int(int d) {
-  const float f = __int_as_float(0x4B400000 + d) - 12582912.0f;
-  return __float_as_uint(f) >> 16;
-}
-
 // S * 2^e2 as the nearest double (ties to even), 0 below the normal range: integer
 // construction, no FP64 arithmetic and no branches, so that the conversions of
 // a thread's elements overlap.
@@ -181,8 +175,6 @@ __device__ inline double oz_to_double(long long S, int e2) {
 
 // ------------------------------------------------------------ slicing
 
-// Both passes run one thread per (row, chunk, lane j): a kCoreK-lane group per
-// row, lane j owning K elements 8j..8j+7 of the chunk (blockIdx.y = chunk).
 // Element (r, k) of the operand is X[r*s_r + (k % KR)*s_k1 + (k / KR)*s_k2].
 struct OzSrc {
   const double* X;
@@ -193,72 +185,146 @@ struct OzSrc {
   long long s_r2;
   int PN;             // > 0: pair-packed symmetric PN x PN matrices, s_r2 apart:
                       // row r = (matrix r / PN, mu = r % PN), column k = nu
+  int vec;            // 8-element runs are contiguous, 16-byte aligned and whole or empty
 };
 
-__device__ inline double oz_load(const OzSrc& S, int r, int k) {
-  if (r >= S.rows || k >= S.K) return 0.0;
-  if (S.PN > 0) {
+// The elements k0 .. k0+7 of row r (zero outside the operand).
+__device__ inline void oz_load8(const OzSrc& S, int r, int k0, double (&x)[8]) {
+  if (r >= S.rows || k0 >= S.K) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = 0.0;
+  } else if (S.PN > 0) {
+    const double* p = S.X + (long long)(r / S.PN) * S.s_r2;
     const int mu = r % S.PN;
-    const long long a = mu > k ? mu : k, b = mu > k ? k : mu;
-    return S.X[(long long)(r / S.PN) * S.s_r2 + a * (a + 1) / 2 + b];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int k = k0 + e, a = max(mu, k), b = min(mu, k);
+      x[e] = k < S.K ? p[(long long)a * (a + 1) / 2 + b] : 0.0;
+    }
+  } else {
+    int q = 0, m = k0;
+    if (S.KR < S.K) {
+      q = k0 / S.KR;
+      m = k0 - q * S.KR;
+    }
+    const double* p = S.X + (S.RR > 0 ? (long long)(r % S.RR) * S.s_r + (long long)(r / S.RR) * S.s_r2
+                                      : (long long)r * S.s_r);
+    if (S.vec) {
+      const double2* v = reinterpret_cast<const double2*>(p + (long long)q * S.s_k2 + m);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const double2 t = v[e];
+        x[2 * e] = t.x;
+        x[2 * e + 1] = t.y;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        x[e] = k0 + e < S.K ? p[(long long)q * S.s_k2 + (long long)m * S.s_k1] : 0.0;
+        if (++m == S.KR) {
+          m = 0;
+          ++q;
+        }
+      }
+    }
   }
-  const int q = k / S.KR, m = k - q * S.KR;
-  const long long ro = S.RR > 0 ? (long long)(r % S.RR) * S.s_r + (long long)(r / S.RR) * S.s_r2 : (long long)r * S.s_r;
-  return S.X[ro + (long long)m * S.s_k1 + (long long)q * S.s_k2];
 }
 
-// exps[r * nkb + kb] = largest biased exponent of row r over K block kb
-// (exps zeroed before; atomicMax is order-independent).
-__global__ void __launch_bounds__(kOzThreads) oz_emax_kernel(OzSrc S, int kb_chunks, int nkb, int* __restrict__ exps) {
-  const int tid = threadIdx.x;
-  const int r = blockIdx.x * (kOzThreads / kCoreK) + tid / kCoreK;
-  const int j = tid % kCoreK;
-  const int c = blockIdx.y;
-  int emax = 0;
+__device__ inline int oz_emax8(const double (&x)[8]) {
+  int e = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) e = max(e, (__double2hiint(x[i]) >> 20) & 0x7FF);
+  return e;
+}
+
+// The digits of eight elements, 16 bytes per plane (planes kPlaneElems apart).  With
+// q_t = V / 2^(48 - 8t) rounded half up, digit t is q_t - 256 q_{t-1}, in 32-bit
+// arithmetic modulo 2^32; 0x4B400000 + d is the FP32 number 1.5 2^23 + d, and the
+// upper half of the difference to 1.5 2^23 is the BF16.
+__device__ inline void oz_digits8(const double (&x)[8], int emax, int smax, uint16_t* dst) {
+  uint32_t lo[8], hi[8], prev[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
-    const double x = oz_load(S, r, c * kOzChunk + 8 * j + e);
-    emax = max(emax, (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7FF));
+    const unsigned long long V = (unsigned long long)oz_fixed(x[e], emax);
+    lo[e] = (uint32_t)V;
+    hi[e] = (uint32_t)(V >> 32);
+    prev[e] = 0u;
   }
 #pragma unroll
-  for (int o = 1; o < kCoreK; o <<= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-  if (j == 0 && r < S.rows && emax > 0) atomicMax(exps + (size_t)r * nkb + c / kb_chunks, emax);
+  for (int t = 0; t < kOzMaxDigits; ++t) {
+    if (t >= smax) break;
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      uint32_t q;
+      if (t == 0) q = (uint32_t)((int)(hi[e] + 0x8000u) >> 16);
+      else if (t == 1) q = (uint32_t)((int)(hi[e] + 0x80u) >> 8);
+      else if (t == 2) q = hi[e] + (lo[e] >> 31);
+      else if (t < 6) q = __funnelshift_r(lo[e], hi[e], 48 - 8 * t) + ((lo[e] >> (47 - 8 * t)) & 1u);
+      else q = lo[e];
+      const uint32_t d = q - 256u * prev[e];
+      prev[e] = q;
+      w[e] = __float_as_uint(__uint_as_float(0x4B400000u + d) - 12582912.0f);
+    }
+    *reinterpret_cast<uint4*>(dst + (size_t)t * kPlaneElems) =
+        make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632), __byte_perm(w[4], w[5], 0x7632),
+                   __byte_perm(w[6], w[7], 0x7632));
+  }
 }
 
-// The digits of chunk c of row r relative to its block exponent.
+// Exponents and digit planes of one K block (blockIdx.y) in one launch: a warp holds
+// eight rows of one chunk (lane = row, 8-element run j: its stores of a digit are
+// 512 contiguous bytes), `slots` warps of the block share the same rows and step
+// through the block's chunks, and exchange their exponents through shared memory.
+// The first kHeld chunks of a warp stay in registers, the others are read again
+// (from L1 or L2).  exps[r * nkb + kb] = largest biased exponent of row r over
+// K block kb.  Bound by the store of the planes (14 bytes an element at 7 digits).
+// Two passes over memory before: exponents by atomicMax into a zeroed array, then
+// the digits, 76 + 194 us for 162816 x 192.
+constexpr int kHeld = 2;
+
 __global__ void __launch_bounds__(kOzThreads) oz_slice_kernel(OzSrc S, int kchunks, int smax, int kb_chunks, int nkb,
-                                                              const int* __restrict__ exps,
+                                                              int slots, int* __restrict__ exps,
                                                               uint16_t* __restrict__ planes) {
-  const int tid = threadIdx.x;
-  const int r = blockIdx.x * (kOzThreads / kCoreK) + tid / kCoreK;
-  const int j = tid % kCoreK;
-  const int c = blockIdx.y;
-  const int emax = exps[(size_t)r * nkb + c / kb_chunks];
-  long long V[8];
+  constexpr int kWarps = kOzThreads / 32;
+  __shared__ int se[kWarps][8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int slot = warp % slots, rg = warp / slots;
+  const int r = (blockIdx.x * (kWarps / slots) + rg) * 8 + (lane >> 2);
+  const int j = lane & 3;
+  const int kb = blockIdx.y, c0 = kb * kb_chunks + slot, c1 = min((kb + 1) * kb_chunks, kchunks);
+  double x[kHeld][8];
+  int emax = 0;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) V[e] = oz_fixed(oz_load(S, r, c * kOzChunk + 8 * j + e), emax);
-  const int rt = r / kOzTileM, rr = r % kOzTileM;
-  uint16_t* dst =
-      planes + ((size_t)rt * kchunks + c) * smax * kPlaneElems + (rr / 8) * (kCoreK * 64) + j * 64 + (rr % 8) * 8;
-  for (int t = 0; t < smax; ++t) {
-    const int p = 48 - 8 * t;
-    uint32_t w[4];
-#pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-      int d0, d1;
-      if (p > 0) {
-        d0 = (int)((V[e] + (1LL << (p - 1))) >> p);
-        d1 = (int)((V[e + 1] + (1LL << (p - 1))) >> p);
-        V[e] -= (long long)d0 << p;
-        V[e + 1] -= (long long)d1 << p;
-      } else {
-        d0 = (int)V[e];
-        d1 = (int)V[e + 1];
-        V[e] = V[e + 1] = 0;
-      }
-      w[e / 2] = bf16_of_int(d0) | (bf16_of_int(d1) << 16);
+  for (int h = 0; h < kHeld; ++h) {
+    const int c = c0 + h * slots;
+    if (c < c1) {
+      oz_load8(S, r, c * kOzChunk + 8 * j, x[h]);
+      emax = max(emax, oz_emax8(x[h]));
     }
-    *reinterpret_cast<uint4*>(dst + (size_t)t * kPlaneElems) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  for (int c = c0 + kHeld * slots; c < c1; c += slots) {
+    double y[8];
+    oz_load8(S, r, c * kOzChunk + 8 * j, y);
+    emax = max(emax, oz_emax8(y));
+  }
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 1));
+  emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 2));
+  if (j == 0) se[warp][lane >> 2] = emax;
+  __syncthreads();
+  for (int k = 0; k < slots; ++k) emax = max(emax, se[rg * slots + k][lane >> 2]);
+  if (slot == 0 && j == 0) exps[(size_t)r * nkb + kb] = emax;
+  const int rt = r / kOzTileM, rr = r % kOzTileM;
+  uint16_t* dst = planes + (size_t)rt * kchunks * smax * kPlaneElems + (rr / 8) * (kCoreK * 64) + j * 64 + (rr % 8) * 8;
+#pragma unroll
+  for (int h = 0; h < kHeld; ++h) {
+    const int c = c0 + h * slots;
+    if (c < c1) oz_digits8(x[h], emax, smax, dst + (size_t)c * smax * kPlaneElems);
+  }
+  for (int c = c0 + kHeld * slots; c < c1; c += slots) {
+    double y[8];
+    oz_load8(S, r, c * kOzChunk + 8 * j, y);
+    oz_digits8(y, emax, smax, dst + (size_t)c * smax * kPlaneElems);
   }
 }
 
@@ -755,14 +821,16 @@ OzOperand oz_slice(const LaCtx& la, const double* X, int rows, int K, long long 
   if (op.kchunks > 65535) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_slice: K too long");
   if (packed_n > 0 && (K != packed_n || rows % packed_n != 0))
     throw RihfError(RIHF_ERR_INVALID_ARG, "oz_slice: packed rows must be whole matrices");
-  OzSrc S{X, rows, K, s_r, s_k1, s_k2, KR, RR, s_r2, packed_n};
-  dim3 grid(op.rows_pad / (kOzThreads / kCoreK), op.kchunks);
-  RIHF_CUDA(cudaMemsetAsync(exps, 0, sizeof(int) * (size_t)op.rows_pad * op.nkb, la.stream));
-  oz_emax_kernel<<<grid, kOzThreads, 0, la.stream>>>(S, op.kb_chunks, op.nkb, exps);
+  OzSrc S{X, rows, K, s_r, s_k1, s_k2, KR, RR, s_r2, packed_n, 0};
+  auto even = [](long long v) { return v % 2 == 0; };
+  S.vec = packed_n == 0 && s_k1 == 1 && K % 8 == 0 && (KR >= K || (KR % 8 == 0 && even(s_k2))) && even(s_r) &&
+          (RR <= 0 || even(s_r2)) && (uintptr_t)X % 16 == 0;
+  int slots = 1;   // warps that share a row's chunks
+  while (slots < kOzThreads / 32 && slots < op.kb_chunks) slots *= 2;
+  const dim3 grid(op.rows_pad / (8 * (kOzThreads / 32 / slots)), op.nkb);
+  oz_slice_kernel<<<grid, kOzThreads, 0, la.stream>>>(S, op.kchunks, smax, op.kb_chunks, op.nkb, slots, exps, planes);
   RIHF_LAUNCH_CHECK();
-  oz_slice_kernel<<<grid, kOzThreads, 0, la.stream>>>(S, op.kchunks, smax, op.kb_chunks, op.nkb, exps, planes);
-  RIHF_LAUNCH_CHECK();
-  if (la.launches) *la.launches += 2;
+  if (la.launches) *la.launches += 1;
   return op;
 }
 
