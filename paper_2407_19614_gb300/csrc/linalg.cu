@@ -329,12 +329,12 @@ constexpr int CB = 32;
 // reciprocal square root.  Block 0 stores L_kk in Ld (the diagonal block of A
 // is still being read by the other blocks; chol_finish_kernel copies it in).
 // Then the panel rows r >= k + b solve y L_kk^T = a_r by forward substitution,
-// four lanes per row (eight rows per warp) splitting each dot product.
+// eight lanes a row as in trsv_lanes_kernel.  (Four lanes a row, each entry a dot
+// product reduced by shuffles, made the rows 2/3 of the step's 34 us.)
 __global__ void __launch_bounds__(128) chol_step_kernel(double* A, int n, int k, int b, int* flag, double* Ld) {
   __shared__ double l[CB][CB + 1];
   __shared__ double piv[2][CB];
   __shared__ double rd[CB];
-  __shared__ double ys[4][8][CB + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double a[CB / 4];
 #pragma unroll
@@ -373,26 +373,27 @@ __global__ void __launch_bounds__(128) chol_step_kernel(double* A, int n, int k,
     if (blockIdx.x == 0 && lane < b && c < b) Ld[(size_t)(k + lane) * CB + c] = a[t];
   }
   __syncthreads();
-  if (threadIdx.x < CB) rd[threadIdx.x] = threadIdx.x < b ? 1.0 / l[threadIdx.x][threadIdx.x] : 0.0;
+  if (threadIdx.x < CB) {
+    rd[threadIdx.x] = threadIdx.x < b ? 1.0 / l[threadIdx.x][threadIdx.x] : 0.0;
+    l[threadIdx.x][threadIdx.x] = 0.0;   // entries that are done subtract zero
+  }
   __syncthreads();
-  const int rs = lane >> 2, sub = lane & 3;
-  double* y = ys[w][rs];
-  for (int r0 = k + b + (blockIdx.x * 4 + w) * 8; r0 < n; r0 += gridDim.x * 32) {
-    const int r = r0 + rs;
-    const bool valid = r < n;
-    for (int i = sub; i < b; i += 4) y[i] = valid ? A[(size_t)r * n + k + i] : 0.0;
-    __syncwarp();
-    for (int i = 0; i < b; ++i) {
-      double part = sub == 0 ? y[i] : 0.0;
-      for (int q = sub; q < i; q += 4) part = fma(-l[i][q], y[q], part);
-      part += __shfl_xor_sync(0xffffffffu, part, 1);
-      part += __shfl_xor_sync(0xffffffffu, part, 2);
-      if (sub == 0) y[i] = part * rd[i];
-      __syncwarp();
+  const int s = lane & 7;
+  for (int r0 = k + b + (blockIdx.x * 4 + w) * 4; r0 < n; r0 += gridDim.x * 16) {
+    const int r = r0 + (lane >> 3);
+    double y[CB / 8];
+#pragma unroll
+    for (int q = 0; q < CB / 8; ++q) y[q] = r < n && s + 8 * q < b ? A[(size_t)r * n + k + s + 8 * q] : 0.0;
+#pragma unroll
+    for (int i = 0; i < CB; ++i) {
+      const double v = __shfl_sync(0xffffffffu, y[i / 8] * rd[i], i & 7, 8);
+      if (s == (i & 7)) y[i / 8] = v;
+#pragma unroll
+      for (int q = i / 8; q < CB / 8; ++q) y[q] = fma(-l[s + 8 * q][i], v, y[q]);
     }
-    if (valid)
-      for (int i = sub; i < b; i += 4) A[(size_t)r * n + k + i] = y[i];
-    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < CB / 8; ++q)
+      if (r < n && s + 8 * q < b) A[(size_t)r * n + k + s + 8 * q] = y[q];
   }
 }
 
@@ -413,7 +414,8 @@ void cholesky(const LaCtx& la, double* A, int n, double* scratch) {
     int b = std::min(CB, n - k);
     int rest = n - k - b;
     // L_kk, and A[k+b:, k:k+b] <- A[k+b:, k:k+b] L_kk^{-T}
-    chol_step_kernel<<<std::max(1, ceil_div(rest, 32)), 128, 0, la.stream>>>(A, n, k, b, la.flag, Ld);
+    const int blocks = std::max(1, std::min(ceil_div(rest, 16), la.sms));
+    chol_step_kernel<<<blocks, 128, 0, la.stream>>>(A, n, k, b, la.flag, Ld);
     RIHF_LAUNCH_CHECK();
     count(la);
     if (rest <= 0) break;
