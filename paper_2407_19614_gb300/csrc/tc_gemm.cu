@@ -115,13 +115,6 @@ __device__ inline void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 __device__ inline void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // One 32-byte sector of a row (p 32-byte aligned).
-__device__ inline void ld_sector(const double* p, double* v) {
-  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
-               : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
-               : "l"(__cvta_generic_to_global(p))
-               : "memory");
-}
-
 __device__ inline void st_sector(double* p, const double* v) {
   asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)), "d"(v[0]), "d"(v[1]),
                "d"(v[2]), "d"(v[3])
@@ -434,6 +427,10 @@ __device__ inline bool oz_valid(const OzTiling& T, int mt, int nt, int c0, int c
   return true;
 }
 
+// Columns that a drain warp passes through shared memory at a time when it adds to C.
+template <int TN>
+constexpr int kStageCols = TN % 32 == 0 ? 16 : 8;
+
 // The integer in accumulator d (d + 1 digit pairs of at most 2^14 K'(S) each): by an
 // FP32 addition where that stays within 2^22, else by a conversion instruction,
 // which only the slow unit has (16 a clock and SM: the read-out is bound by it).
@@ -669,57 +666,63 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         ++grp;
       }
       if (!ok) break;
-      // all of the thread's values first, then the stores: whole 32-byte sectors
-      // when the row is contiguous and aligned (16-byte halves write a sector twice)
+      // all of the thread's values first, then the stores
       const int nv = min(ncol, T.N - n0);
       double v[ncol];
 #pragma unroll
-      for (int k = 0; k < ncol; ++k) {
+      for (int k = 0; k < ncol; ++k)
         v[k] = oz_to_double(T.aneg ? -acc[k] : acc[k], ea + __shfl_sync(0xffffffffu, eb, k));
-      }
       if (T.scale)   // not a predicate on each product: those hold the FP64 pipe also when it is false
 #pragma unroll
         for (int k = 0; k < ncol; ++k) v[k] *= alpha;
       const int mr = MR < T.M ? (int)MR : T.M;
       double* dst = C + (long long)(m % mr) * cs_m1 + (long long)(m / mr) * cs_m2 + (long long)n0 * cs_n;
+      // whole 32-byte sectors when the row is contiguous and aligned (16-byte halves
+      // write a sector twice)
       const bool sectors =
           __all_sync(0xffffffffu, m >= T.M || (cs_n == 1 && nv == ncol && ((uintptr_t)dst & 31) == 0));
-      if (m < T.M) {
+      if (atomic == 2 && cs_n == 1) {
+        // added to: the warp's 32 rows go through shared memory, W columns at a time,
+        // so that 32 / W whole row segments are read and written at once
+        constexpr int W = kStageCols<TN>, RP = 32 / W;
+        double* stg = reinterpret_cast<double*>(smem + (size_t)T.nst * T.stage_bytes + kBookBytes) + warp * 32 * (W + 1);
+        const int cc = lane % W, rr = lane / W, m0 = mt * kOzTileM + 32 * (warp & 3);
+#pragma unroll
+        for (int k0 = 0; k0 < ncol; k0 += W) {
+          __syncwarp();
+#pragma unroll
+          for (int k = 0; k < W; ++k) stg[lane * (W + 1) + k] = v[k0 + k];
+          __syncwarp();
+          double old[W];
+#pragma unroll
+          for (int i = 0; i < W; ++i) {
+            const int q = i * RP + rr;
+            const double* p =
+                reinterpret_cast<const double*>(__shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)dst, q));
+            old[i] = m0 + q < T.M && k0 + cc < nv ? p[k0 + cc] : 0.0;
+          }
+#pragma unroll
+          for (int i = 0; i < W; ++i) {
+            const int q = i * RP + rr;
+            double* p = reinterpret_cast<double*>(__shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)dst, q));
+            const double sum = old[i] + stg[q * (W + 1) + cc];
+            if (m0 + q < T.M && k0 + cc < nv) p[k0 + cc] = sum;
+          }
+        }
+      } else if (m < T.M) {
         if (atomic == 1) {
 #pragma unroll
           for (int k = 0; k < ncol; ++k)
             if (k < nv) atomicAdd(dst + (long long)k * cs_n, v[k]);
-        } else if (sectors) {
+        } else if (sectors && atomic == 0) {
 #pragma unroll
-          for (int k0 = 0; k0 < ncol; k0 += 8) {   // two sectors in flight at a time
-            if (atomic == 2) {
-              double old[8];
-              ld_sector(dst + k0, old);
-              ld_sector(dst + k0 + 4, old + 4);
-#pragma unroll
-              for (int k = 0; k < 8; ++k) v[k0 + k] = old[k] + v[k0 + k];
-            }
-            st_sector(dst + k0, v + k0);
-            st_sector(dst + k0 + 4, v + k0 + 4);
-          }
+          for (int k0 = 0; k0 < ncol; k0 += 4) st_sector(dst + k0, v + k0);
         } else if (cs_n == 1 && ((uintptr_t)dst & 15) == 0) {
           double2* d2 = reinterpret_cast<double2*>(dst);
 #pragma unroll
-          for (int k0 = 0; k0 < ncol / 2; k0 += 4) {   // four pairs in flight at a time
-            double2 old[4];
-#pragma unroll
-            for (int k = k0; k < k0 + 4; ++k)
-              old[k - k0] = atomic == 2 && 2 * k + 1 < nv ? d2[k] : make_double2(0.0, 0.0);
-#pragma unroll
-            for (int k = k0; k < k0 + 4; ++k) {
-              if (2 * k + 1 < nv) {
-                if (atomic == 2) d2[k] = make_double2(old[k - k0].x + v[2 * k], old[k - k0].y + v[2 * k + 1]);
-                else d2[k] = make_double2(v[2 * k], v[2 * k + 1]);
-              } else if (2 * k < nv) {
-                if (atomic == 2) dst[2 * k] += v[2 * k];
-                else dst[2 * k] = v[2 * k];
-              }
-            }
+          for (int k = 0; k < ncol / 2; ++k) {
+            if (2 * k + 1 < nv) d2[k] = make_double2(v[2 * k], v[2 * k + 1]);
+            else if (2 * k < nv) dst[2 * k] = v[2 * k];
           }
         } else {
 #pragma unroll
@@ -888,7 +891,10 @@ void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   T.kchunks = A.kchunks;
   T.G = std::max(1, (1024 / T.s) / kOzChunk);
   T.stage_bytes = T.s * (kPlaneElems * 2 + T.TN * kOzChunk * 2);
-  T.nst = std::min(kMaxStages, (kSmemMax - kBookBytes - 1024) / T.stage_bytes);
+  // what the drain warps need to add to C row by row
+  const int stage_cols = T.TN % 32 == 0 ? 16 : 8;
+  const int add_bytes = g.accumulate ? kDrainThreads * (stage_cols + 1) * 8 : 0;
+  T.nst = std::min(kMaxStages, (kSmemMax - kBookBytes - 1024 - add_bytes) / T.stage_bytes);
   if (T.nst < 1) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: stage exceeds shared memory");
   // a power of two goes into the integer result instead of an FP64 product
   int aexp = 0;
@@ -897,7 +903,7 @@ void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   T.aexp = pow2 ? aexp - 1 : 0;
   T.aneg = pow2 && g.alpha < 0.0 ? 1 : 0;
   T.scale = pow2 ? 0 : 1;
-  const int smem = std::max(kSmemMin, T.nst * T.stage_bytes + kBookBytes + 1024);
+  const int smem = std::max(kSmemMin, T.nst * T.stage_bytes + kBookBytes + 1024 + add_bytes);
   const OzKernel kernel = oz_kernel(T.s, T.TN);
   raise_smem_limit((const void*)kernel, kSmemMax);
   const int grid = (int)std::min<long long>(nitems, sms);
