@@ -2127,7 +2127,7 @@ static void build_sad(rihf_ctx* c) {
       if (rc != RIHF_OK && rc != RIHF_ERR_NOT_CONVERGED) { c->sad_note = "atomic SCF failed"; return; }
       at.F.resize((size_t)at.na * at.m);
       for (int r = 0; r < at.na; ++r)
-        for (int q = 0; q < at.m; ++q) at.F[(size_t)r * at.m + q] = C[(size_t)r * sub->N + q] * std::sqrt(occ[q]);
+        for (int q = 0; q < at.m; ++q) at.F[(size_t)r * at.m + q] = C[(size_t)r * at.na + q] * std::sqrt(occ[q]);
       if (c->verbose || getenv("RIHF_VERBOSE"))
         fprintf(stderr, "rihf: SAD atom Z=%d: %d functions, %d occupied, E = %.10f (%d iterations)\n", zc, at.na,
                 at.m, e, it);
