@@ -1420,15 +1420,15 @@ static void diagonalise(rihf_ctx* c, const double* Fin, bool warm) {
     // refine-only iterations start from them.  Below max|e| = 0.1 (the first
     // iterations after a nuclear step) two sweeps reach ~1e-5 and one
     // refinement and one re-orthonormalisation step suffice; larger errors
-    // (a cold start) take six sweeps and three refinement steps (three or four
-    // leave the early iterates, and so the path of DIIS, measurably off: with four
-    // the forces of two starts of (H2O)8 at max|e| < 5e-9 differ by 2.1..5.5e-8 over
-    // repeated runs, with six by 1.6..3.7e-8).
+    // (a first iteration) take five sweeps and three refinement steps: fewer leave
+    // the early iterates, and so the path of DIIS, measurably off (forces of two
+    // starts of (H2O)8 at max|e| < 5e-9, 70 runs: the median difference is 2.8e-8 with
+    // four sweeps and 9 runs are above 5e-8; 2.1e-8 with five, one run above).
     const bool light = c->last_err < 0.1;
     graph_or_eager(c, c->diag_graphs[(light ? 4 : 2) + (Fin == c->F ? 0 : 1)], "eigh F' (jacobi+refine)", [&]() {
       form_fp();
       if (light) eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 1, c->Cprev, false, 2, 1);
-      else eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 3, c->Cprev, false, 6);
+      else eigh(la, c->Fp, n, c->eps, c->Cp, c->eigws, 3, c->Cprev, false, 5);
     });
   } else {
     graph_or_eager(c, c->diag_graphs[Fin == c->F ? 0 : 1], "eigh F' (refine only)", [&]() {
