@@ -104,10 +104,10 @@ __device__ inline void mma_commit(uint64_t* bar, uint32_t lead) {
       : "memory");
 }
 
-// 32 lanes x 8 consecutive 32-bit columns; thread i gets lane (base + i).
-__device__ inline void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+// 32 lanes x 4 consecutive 32-bit columns; thread i gets lane (base + i).
+__device__ inline void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr)
                : "memory");
 }
@@ -327,12 +327,12 @@ __global__ void __launch_bounds__(kOzThreads) oz_slice_kernel(OzSrc S, int kchun
 // columns).  Work items are (row tile, column tile, K block) triples taken from
 // a global counter, so tiles that the symmetry options skip cost nothing and
 // the SMs stay balanced.
-//   warp 9 (one lane): takes items, streams their K chunks' digit planes into
+//   warp 17 (one lane): takes items, streams their K chunks' digit planes into
 //     a ring of shared-memory stages with bulk copies;
-//   warp 8: issues the MMAs of each chunk and commits stage releases and, every
+//   warp 16: issues the MMAs of each chunk and commits stage releases and, every
 //     G chunks, a full accumulator group;
-//   warps 0-7: drain the s TMEM accumulators of each group (a row and half the
-//     columns per thread) into int64 fixed-point sums; the group is released when
+//   warps 0-15: drain the s TMEM accumulators of each group (a row and a quarter
+//     of the columns per thread) into int64 fixed-point sums; the group is released when
 //     its last columns are in registers, so the next group's MMAs overlap the
 //     rest of the conversion and, at a tile's end, the stores.
 // The kernel is compiled per digit count and column tile: every descriptor offset
@@ -350,8 +350,12 @@ __global__ void __launch_bounds__(kOzThreads) oz_slice_kernel(OzSrc S, int kchun
 // leave, the copies and MMAs still in flight are awaited (bounded) and
 // la.flag[1] is set.
 
-constexpr int kGemmThreads = 320;
-constexpr int kDrainThreads = 256;
+// Four drain warps a scheduler: the read-out and the epilogue are chains of integer
+// instructions that two warps did not cover (a gradient's Y at 580 orbitals, whose
+// tiles are two chunks long and all epilogue, 8.9 -> 8.3 ms; K at 384 orbitals 3 to 5 %).
+constexpr int kDrainThreads = 512;
+constexpr int kMmaWarp = kDrainThreads / 32, kCopyWarp = kMmaWarp + 1;
+constexpr int kGemmThreads = kDrainThreads + 64;
 constexpr int kMaxStages = 4;
 constexpr int kItemSlots = 2;
 constexpr int kTmemCols = 512;
@@ -429,7 +433,7 @@ __device__ inline bool oz_valid(const OzTiling& T, int mt, int nt, int c0, int c
 
 // Columns that a drain warp passes through shared memory at a time when it adds to C.
 template <int TN>
-constexpr int kStageCols = TN % 32 == 0 ? 16 : 8;
+constexpr int kStageCols = TN % 32 == 0 ? 8 : 4;
 
 // The integer in accumulator d (d + 1 digit pairs of at most 2^14 K'(S) each): by an
 // FP32 addition where that stays within 2^22, else by a conversion instruction,
@@ -469,13 +473,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     bk->issued = bk->consumed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 8) tmem_alloc(&bk->tslot, kTmemCols);
+  if (warp == kMmaWarp) tmem_alloc(&bk->tslot, kTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t taddr = bk->tslot;
 
-  if (warp == 9) {
+  if (warp == kCopyWarp) {
     if (lane == 0) {   // ---------------- producer
       uint32_t i = 0;
       bool ok = true;
@@ -520,7 +524,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       }
     }
     __syncwarp();
-  } else if (warp == 8) {
+  } else if (warp == kMmaWarp) {
     // ---------------- MMA issuer: the warp stays converged, lane 0 issues
     // BF16 x BF16 -> FP32, M = 128; N is set per MMA
     const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kOzTileM >> 4) << 24);
@@ -594,16 +598,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (lane == 0) bk->consumed = (int)i;
     if (*abort && last_st >= 0) mbar_wait(&bk->empty[last_st], last_par);   // MMAs in flight
     __syncwarp();
-  } else {   // ---------------- drain: warps 0-7
+  } else {   // ---------------- drain: warps 0-15
     const int row = 32 * (warp & 3) + lane;
-    constexpr int ncol = TN / 2;
+    constexpr int ncol = TN / 4;   // a row and a quarter of the columns per thread
     const int col0 = (warp >> 2) * ncol;
     const uint32_t t_row = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
     // one thread polls, the other drain threads wait on a hardware named
     // barrier (spinning 256 threads would compete with the copy and MMA
     // threads for issue slots and for the barrier unit); the poller is lane 0
-    // of warp 2, on a scheduler that neither the MMA warp (8) nor the copy
-    // warp (9) uses
+    // of warp 2, on a scheduler that neither the MMA nor the copy warp uses
     int nwait = 0;
     auto drain_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
       const int k = nwait++ & 1;
@@ -623,7 +626,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       int mt, nt, split, c0, c1;
       oz_decode(T, idx, mt, nt, split, c0, c1);
       // the exponents (padded to whole tiles) are fetched ahead of their use:
-      // lane k's eb is that of column k of the warp's ncol <= 32
+      // lane k's eb is that of column k of the warp's ncol <= 16
       const int m = mt * kOzTileM + row, n0 = nt * TN + col0;
       const int ea = A.exps[(size_t)m * A.nkb + split] - 2095 + T.aexp;
       const int eb = lane < ncol ? B.exps[(size_t)(n0 + lane) * B.nkb + split] : 0;
@@ -634,23 +637,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         ok = drain_wait(&bk->accfull, grp & 1);
         if (!ok) break;
         tc_fence_after();
-        // eight columns of all s diagonals at a time (the warp's last block read
+        // four columns of all s diagonals at a time (the warp's last block read
         // frees the accumulators): the element's sum then has constant weights
         // 2^37, 2^29, ... 2^-11, one multiply-add each
 #pragma unroll
-        for (int q8 = 0; q8 < ncol / 8; ++q8) {
-          uint32_t r[S][8];
+        for (int q4 = 0; q4 < ncol / 4; ++q4) {
+          uint32_t r[S][4];
 #pragma unroll
-          for (int d = 0; d < S; ++d) tmem_ld8(t_row + (uint32_t)(d * TN + col0 + 8 * q8), r[d]);
+          for (int d = 0; d < S; ++d) tmem_ld4(t_row + (uint32_t)(d * TN + col0 + 4 * q4), r[d]);
           tmem_wait_ld();
-          if (q8 == ncol / 8 - 1) {
+          if (q4 == ncol / 4 - 1) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bk->accempty);
           }
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            long long a = acc[8 * q8 + e];
+          for (int e = 0; e < 4; ++e) {
+            long long a = acc[4 * q4 + e];
             int low = 0;
 #pragma unroll
             for (int d = 0; d < S; ++d) {
@@ -660,7 +663,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
               else low += v >> (sh < 0 ? -sh : 0);
             }
             if (S > 5) a += low;
-            acc[8 * q8 + e] = a;
+            acc[4 * q4 + e] = a;
           }
         }
         ++grp;
@@ -740,7 +743,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 
   __syncthreads();
   if (*abort) {
-    if (warp == 9 && lane == 0) {
+    if (warp == kCopyWarp && lane == 0) {
       // copies still in flight: chunks issued but never consumed
       for (int i = bk->consumed; i < bk->issued; ++i) mbar_wait(&bk->full[i % T.nst], (i / T.nst) & 1);
     }
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == kMmaWarp) {
     tc_fence_after();
     tmem_dealloc(taddr, kTmemCols);
   }
@@ -892,7 +895,7 @@ void oz_gemm(const LaCtx& la, const OzGemmArgs& g) {
   T.G = std::max(1, (1024 / T.s) / kOzChunk);
   T.stage_bytes = T.s * (kPlaneElems * 2 + T.TN * kOzChunk * 2);
   // what the drain warps need to add to C row by row
-  const int stage_cols = T.TN % 32 == 0 ? 16 : 8;
+  const int stage_cols = T.TN % 32 == 0 ? 8 : 4;
   const int add_bytes = g.accumulate ? kDrainThreads * (stage_cols + 1) * 8 : 0;
   T.nst = std::min(kMaxStages, (kSmemMax - kBookBytes - 1024 - add_bytes) / T.stage_bytes);
   if (T.nst < 1) throw RihfError(RIHF_ERR_INVALID_ARG, "oz_gemm: stage exceeds shared memory");
