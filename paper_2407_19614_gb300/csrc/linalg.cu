@@ -1083,7 +1083,7 @@ void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double*
     dgemm(la, g);
     RIHF_CUDA(cudaMemcpyAsync(V, XE, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, la.stream));
   }
-  }   // one-CTA Jacobi
+  }   // Jacobi
   for (int it = 0; it < refine; ++it) {
     GemmArgs gr;   // R = V^T V
     gr.M = n; gr.N = n; gr.K = n; gr.A = V; gr.lda = n; gr.transA = true; gr.B = V; gr.ldb = n; gr.C = R; gr.ldc = n;

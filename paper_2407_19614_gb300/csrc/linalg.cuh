@@ -90,7 +90,7 @@ void trsm_lower(const LaCtx& la, const double* L, int n, double* X, long long nc
 
 // Symmetric eigen-decomposition of an n x n FP64 matrix A (row-major):
 // W (n, ascending) and V (n x n, column k = eigenvector k).  Up to order
-// kJacobiMax FP32 parallel Jacobi in one CTA, above it the FP64 tridiagonal
+// kJacobiMax FP32 parallel Jacobi in a cluster of CTAs, above it the FP64 tridiagonal
 // path (eigh_tridiag.cuh; Vguess is of no use to it), then Ogita-Aishima
 // refinement in FP64 (`refine` steps; at most kTridiagRefine after the
 // tridiagonal path, whose vectors are FP64 already).
