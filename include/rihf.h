@@ -322,6 +322,21 @@ int rihf_learn_params(rihf_ctx* ctx, float* out);
 int rihf_mlp_eval(int hidden, int M, const float* params, const float* X, const float* t, float lr, int iters,
                   float* y, float* grad, float* params_out, float* loss2, float* losses, int device);
 
+/* Fault injection for tests of a caller's error handling: the context's next
+   device wait at `point` is reported as run out, so that the call it belongs to
+   (rihf_update_geometry; rihf_scf for GUESS, ITERATION and, with guess 3 or 4,
+   HISTORY; rihf_gradient) returns RIHF_ERR_TIMEOUT.  No kernel waits or
+   fails: the host sets the status word that an expired wait would set.  One
+   shot.  Errors: INVALID_ARG. */
+enum rihf_wait_point {
+  RIHF_WAIT_FIT = 1,
+  RIHF_WAIT_GUESS = 2,
+  RIHF_WAIT_ITERATION = 3,
+  RIHF_WAIT_HISTORY = 4,
+  RIHF_WAIT_GRADIENT = 5
+};
+int rihf_inject_timeout(rihf_ctx* ctx, int point);
+
 const char* rihf_strerror(int code);
 const char* rihf_last_error(void);
 void rihf_destroy(rihf_ctx* ctx);

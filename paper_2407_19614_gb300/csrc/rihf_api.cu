@@ -661,6 +661,7 @@ struct rihf_ctx {
   double last_err = 1.0;   // max|e| of the latest SCF iteration
   double prev_err = 1.0;   // and of the one before
   bool force_cold = false; // next diagonalisation: full Jacobi from scratch (SCF stall recovery)
+  int inject = 0;          // point at which the next wait is reported as run out (rihf_inject_timeout)
   double timings[5] = {0, 0, 0, 0, 0};
   cudaEvent_t ev[8];
 
@@ -812,6 +813,28 @@ static void eri3_all(rihf_ctx* c, double* T) {
   else launch_eri3(c->ic(), c->prim(), c->aux(), c->d_pairs, c->ptab(), c->groups, kTaskGroups, T);
 }
 
+// Bounded device waits (the digit-plane GEMM's, the tridiagonalisation's grid
+// barriers) raise d_flag[1] when they run out, and what follows them is garbage.  Every
+// entry point that can launch one looks at the mark after its last launch and nobody
+// clears it in between.  late_clear: the mark was read and is being reported.
+static void late_clear(rihf_ctx* c) { RIHF_CUDA(cudaMemsetAsync(c->d_flag + 1, 0, sizeof(int), c->stream)); }
+
+// Reads (waiting for the stream) and clears the mark.
+static bool late_take(rihf_ctx* c) {
+  int late = 0;
+  RIHF_CUDA(cudaMemcpyAsync(&late, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  RIHF_CUDA(cudaStreamSynchronize(c->stream));
+  if (late) late_clear(c);
+  return late != 0;
+}
+
+// Host-side fault injection: raises the mark here if the caller asked for this point.
+static void inject_late(rihf_ctx* c, int point) {
+  if (c->inject != point) return;
+  c->inject = 0;
+  RIHF_CUDA(cudaMemsetAsync(c->d_flag + 1, 1, sizeof(int), c->stream));
+}
+
 // Geometry-dependent part of setup: shell centres, one-electron, metric,
 // Cholesky, 3-centre integrals, fit, orthogonaliser.
 static void compute_geometry_rest(rihf_ctx* c);
@@ -928,10 +951,16 @@ static void compute_geometry_rest(rihf_ctx* c) {
     unpack_sym_batch(la, c->Bp, NA, N, c->npp, c->Bu);
     c->bu_is_B = true;
   }
-  int flag = 0;
-  RIHF_CUDA(cudaMemcpyAsync(&flag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  inject_late(c, RIHF_WAIT_FIT);
+  int flag[2] = {0, 0};
+  auto late = [&]() {
+    late_clear(c);
+    throw RihfError(RIHF_ERR_TIMEOUT, "fit and orthogonaliser: a bounded device wait ran out");
+  };
+  RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
   RIHF_CUDA(cudaStreamSynchronize(s));
-  if (flag) throw RihfError(RIHF_ERR_NOT_POSITIVE_DEFINITE, "metric (P|Q) is not positive definite");
+  if (flag[1]) late();
+  if (flag[0]) throw RihfError(RIHF_ERR_NOT_POSITIVE_DEFINITE, "metric (P|Q) is not positive definite");
   // Orthogonaliser.  First try X = L_S^{-T} (S = L_S L_S^T); since
   // lambda_min(S) >= 1 / Tr(S^{-1}) = 1 / ||L_S^{-1}||_F^2, a bound above
   // lindep_tau proves that canonical orthogonalisation would drop nothing, and
@@ -947,9 +976,10 @@ static void compute_geometry_rest(rihf_ctx* c) {
     dot(la, N * N, c->T1, c->T1, c->scal + 3);
     double tr = 0.0;
     RIHF_CUDA(cudaMemcpyAsync(&tr, c->scal + 3, sizeof(double), cudaMemcpyDeviceToHost, s));
-    RIHF_CUDA(cudaMemcpyAsync(&flag, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+    RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaStreamSynchronize(s));
-    chol_ok = !flag && std::isfinite(tr) && tr > 0.0 && 1.0 / tr > c->opt.lindep_tau;
+    if (flag[1]) late();
+    chol_ok = !flag[0] && std::isfinite(tr) && tr > 0.0 && 1.0 / tr > c->opt.lindep_tau;
     RIHF_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), s));
   }
   std::vector<double> sw;
@@ -958,10 +988,9 @@ static void compute_geometry_rest(rihf_ctx* c) {
     eigh(la, c->S, N, c->Sw, c->Sv, c->eigws, 4, nullptr);
     sw.resize(N);
     RIHF_CUDA(cudaMemcpyAsync(sw.data(), c->Sw, sizeof(double) * N, cudaMemcpyDeviceToHost, s));
-    int late = 0;
-    RIHF_CUDA(cudaMemcpyAsync(&late, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+    RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
     RIHF_CUDA(cudaStreamSynchronize(s));
-    if (late) throw RihfError(RIHF_ERR_TIMEOUT, "overlap eigenvalues: a bounded device wait ran out");
+    if (flag[1]) late();
     while (k0 < N && sw[k0] <= c->opt.lindep_tau) ++k0;
     if (k0 == N) throw RihfError(RIHF_ERR_NOT_POSITIVE_DEFINITE, "overlap matrix has no eigenvalue above lindep_tau");
   }
@@ -1020,7 +1049,9 @@ static void compute_geometry_rest(rihf_ctx* c) {
     RIHF_CUDA(cudaMemcpyAsync(c->Xo, c->T1, sizeof(double) * N * nind, cudaMemcpyDeviceToDevice, s));
   }
   cudaEventRecord(c->ev[1], s);
+  RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
   RIHF_CUDA(cudaStreamSynchronize(s));
+  if (flag[1]) late();
   c->tracer.flush();
   float ms = 0.f;
   cudaEventElapsedTime(&ms, c->ev[0], c->ev[1]);
@@ -2217,6 +2248,14 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
   const size_t n2 = (size_t)N * N;
   cudaStream_t s = c->stream;
   c->timings[1] = c->timings[2] = 0.0;
+  // the guess may already wait on the device (a diagonalisation of H, Loewdin factors):
+  // the mark is cleared before it and read once after the last iteration
+  late_clear(c);
+  auto late = [&]() {
+    late_clear(c);
+    c->converged = c->have_orbitals = c->have_cprev = false;   // whatever they hold came after the wait
+    throw RihfError(RIHF_ERR_TIMEOUT, "SCF: a bounded device wait ran out");
+  };
   cudaEventRecord(c->ev[7], s);   // SCF start (diagonalisation time = total - builds)
   if (!c->Bz.planes && c->pc == c->NA && !c->bu_is_B) {
     // FP64 mode holds all of B expanded in Bu, which the captured Fock-build
@@ -2333,6 +2372,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     c->last_guess = 0;
     c->pending_example = false;
   }
+  inject_late(c, RIHF_WAIT_GUESS);
   const bool sad_first = c->last_guess == 5;
   const int size = c->opt.diis_size;
   double E = 0.0, Eold = 0.0, emax = 0.0;
@@ -2363,7 +2403,6 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
   int since_best = 0, dbase = 0;
   c->tc_builds = 0;
   c->confirm_builds = 0;
-  RIHF_CUDA(cudaMemsetAsync(c->d_flag + 1, 0, sizeof(int), s));
   for (it = 1; it <= c->opt.max_iter; ++it) {
     cudaEventRecord(c->ev[2], s);
     const bool full = fp64_next;
@@ -2385,6 +2424,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     } else {
       fock_and_error(c, variant);
     }
+    inject_late(c, RIHF_WAIT_ITERATION);
     cudaEventRecord(c->ev[3], s);
     int slot = (it - 1 - dbase) % size;
     int m = std::min(it - dbase, size);
@@ -2398,6 +2438,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
     c->prev_err = c->last_err;
     c->last_err = emax;
     if (c->verbose || getenv("RIHF_VERBOSE")) fprintf(stderr, "rihf_scf it %3d  E = %.12f  max|e| = %.3e  dE = %.3e\n", it, E, emax, E - Eold);
+    if (!std::isfinite(E) && late_take(c)) late();
     if (!std::isfinite(E)) throw RihfError(RIHF_ERR_NOT_CONVERGED, "SCF energy is not finite");
     const bool crit = it > 1 && std::fabs(E - Eold) < c->opt.conv_e && emax < c->opt.conv_diis;
     emax_prev = emax;
@@ -2466,8 +2507,16 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
   cudaEventElapsedTime(&ms, c->ev[7], c->ev[4]);
   c->timings[2] = std::max(0.0, (double)ms - c->timings[1]);
   c->tracer.flush();
-  if (tc_flag) throw RihfError(RIHF_ERR_TIMEOUT, "tensor-core RI-K: a bounded device wait ran out");
-  if (conv) learn_and_push_history(c);
+  if (tc_flag) late();
+  if (conv) {
+    learn_and_push_history(c);
+    inject_late(c, RIHF_WAIT_HISTORY);
+    if (c->hist_lowdin && late_take(c)) {   // the SCF's own results stand
+      c->nhist = 0;
+      c->lowdin_serial = -1;
+      throw RihfError(RIHF_ERR_TIMEOUT, "guess history: a bounded device wait ran out");
+    }
+  }
   if (energy) *energy = E;
   if (iters) *iters = it;
   c->last_iters = it;
@@ -2661,6 +2710,7 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   { TraceScope t(c->tracer, s, "grad_eri2_kernel (fused d(P|Q) . Z)", (double)NA * NA * 8, 1);
     if (c->opt.pure) launch_lane_grad_eri2(ic, c->aux(), c->lane_eri2, c->d_ket, c->Zm, g_two);
     else launch_grad_eri2(ic, c->aux(), c->max_la, c->Zm, g_two); }
+  inject_late(c, RIHF_WAIT_GRADIENT);
 }
 
 // Per-atom parts back to the host, nuclear repulsion, the sum.
@@ -2670,9 +2720,15 @@ static void gradient_finish(rihf_ctx* c, double* grad) {
   c->grad_parts_h.assign(15 * nat, 0.0);
   RIHF_CUDA(cudaMemcpyAsync(c->grad_parts_h.data(), c->grad_parts, sizeof(double) * 12 * nat,
                             cudaMemcpyDeviceToHost, s));
+  int late = 0;
+  RIHF_CUDA(cudaMemcpyAsync(&late, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   cudaEventRecord(c->ev[6], s);
   RIHF_CUDA(cudaStreamSynchronize(s));
   c->tracer.flush();
+  if (late) {
+    late_clear(c);
+    throw RihfError(RIHF_ERR_TIMEOUT, "gradient: a bounded device wait ran out");
+  }
   float ms = 0.f;
   cudaEventElapsedTime(&ms, c->ev[5], c->ev[6]);
   c->timings[3] = ms;
@@ -2709,6 +2765,12 @@ int rihf_gradient(rihf_ctx* c, double* grad) {
   RIHF_API_END
 }
 
+int rihf_inject_timeout(rihf_ctx* c, int point) {
+  if (!c || point < RIHF_WAIT_FIT || point > RIHF_WAIT_GRADIENT) return RIHF_ERR_INVALID_ARG;
+  c->inject = point;
+  return RIHF_OK;
+}
+
 int rihf_query(rihf_ctx* c, int* N, int* Naux, int* nocc, int* natoms) {
   if (!c) return RIHF_ERR_INVALID_ARG;
   if (N) *N = c->N;
@@ -2737,7 +2799,7 @@ int rihf_get_matrix(rihf_ctx* c, int which, double* out) {
         LaCtx la = c->la();
         identity(la, c->Linv, c->NA);
         trsm_lower(la, c->L, c->NA, c->Linv, c->NA, false, 0, c->trsm_tmp);
-        RIHF_CUDA(cudaStreamSynchronize(c->stream));
+        if (late_take(c)) throw RihfError(RIHF_ERR_TIMEOUT, "inverse factor: a bounded device wait ran out");
         c->have_linv = true;
       }
       RIHF_CUDA(cudaMemcpy(out, c->Linv, na2 * 8, cudaMemcpyDeviceToHost));

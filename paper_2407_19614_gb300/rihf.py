@@ -21,6 +21,7 @@ ERRORS = {-1: "INVALID_ARG", -2: "OOM", -3: "CUDA", -4: "NOT_CONVERGED", -5: "TI
 MAT = dict(S=0, H=1, A=2, LINV=3, T3=4, B=5, J=6, K=7, F=8, D=9, GRAD_PARTS=10, SCHWARZ=11, DPRED=12, FEATURES=13,
            DSAD=14)
 PRECISION_FP64, PRECISION_MIXED = 0, 1
+WAIT = dict(FIT=1, GUESS=2, ITERATION=3, HISTORY=4, GRADIENT=5)
 
 
 class RihfError(RuntimeError):
@@ -46,7 +47,7 @@ EXPORTS = ["rihf_default_options", "rihf_setup", "rihf_update_geometry", "rihf_s
            "rihf_query", "rihf_get_matrix", "rihf_screening_stats", "rihf_timings", "rihf_strerror",
            "rihf_last_error", "rihf_destroy", "rihf_eigh", "rihf_stream", "rihf_trace", "rihf_trace_stats",
            "rihf_scf_stats", "rihf_eigh_noalloc", "rihf_tc_dgemm", "rihf_learn_config", "rihf_learn_stats",
-           "rihf_mlp_eval", "rihf_learn_params", "rihf_batch_step"]
+           "rihf_mlp_eval", "rihf_learn_params", "rihf_batch_step", "rihf_inject_timeout"]
 
 _lib = None
 
@@ -99,6 +100,8 @@ def load(path: str = LIB_PATH):
     lib.rihf_learn_params.restype = I
     lib.rihf_batch_step.argtypes = [I, P, P, I, P, P, P, I]
     lib.rihf_batch_step.restype = I
+    lib.rihf_inject_timeout.argtypes = [P, I]
+    lib.rihf_inject_timeout.restype = I
     lib.rihf_destroy.argtypes = [P]
     lib.rihf_destroy.restype = None
     for name in ("rihf_setup", "rihf_update_geometry", "rihf_scf", "rihf_gradient", "rihf_query",
@@ -270,6 +273,10 @@ class Context:
         out = np.zeros(n, dtype=np.float32)
         _check(self.lib.rihf_learn_params(self.h, _p(out)))
         return out
+
+    def inject_timeout(self, point):
+        """Report the next device wait at `point` (a key of WAIT) as run out (no kernel waits or fails)."""
+        _check(self.lib.rihf_inject_timeout(self.h, WAIT[point]))
 
     def update_geometry(self, xyz):
         x = np.ascontiguousarray(xyz, dtype=np.float64)
