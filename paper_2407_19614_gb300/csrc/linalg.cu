@@ -681,7 +681,10 @@ void trsm_lower_t_tc(const LaCtx& la, const double* L, int n, double* X, long lo
 // One-sided (Hestenes) Jacobi in FP32: with B = A + sigma I positive definite
 // (sigma from a Gershgorin bound), column rotations U <- U J drive the columns of
 // U = B V to mutual orthogonality; then v_j = u_j / |u_j| and lambda_j = |u_j| -
-// sigma.  Only U (n x n, column-major) is stored.
+// sigma.  Only U (n x n, column-major) is stored.  A is scaled by the power of two
+// that brings its largest row sum into [1, 2) (which changes no rounding): unscaled,
+// the fourth powers of the entries that the convergence test multiplies leave the FP32
+// range at norms below 1e-10 and above 1e10.
 //
 // The columns form nb blocks of H (nb even); in a round a warp holds the two
 // blocks of one block pair in registers (R rows of every column per lane) and
@@ -742,9 +745,12 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : 32 * 4)
   float top = red[32];
   if constexpr (CL > 1)
     for (int q = 0; q < CL; ++q) top = fmaxf(top, *cg::this_cluster().map_shared_rank(red + 32, q));
-  const float sigma = 1.05f * top + 1e-20f;
+  const int ex = min(max((__float_as_int(top) >> 23) - 127, -126), 126);   // top >= 0
+  const float down = __int_as_float((127 - ex) << 23), up = __int_as_float((127 + ex) << 23);   // 2^-ex, 2^ex
+  const float sigma = 1.05f * (top * down) + 1e-20f;
   for (int j = gw; j < n; j += nw)
-    for (int i = lane; i < n; i += 32) st(U + (size_t)j * n + i, (float)A[(size_t)i * n + j] + (i == j ? sigma : 0.f));
+    for (int i = lane; i < n; i += 32)
+      st(U + (size_t)j * n + i, (float)A[(size_t)i * n + j] * down + (i == j ? sigma : 0.f));
   sync();
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     if (threadIdx.x == 0) flag = 0;
@@ -845,7 +851,7 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : 32 * 4)
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     const float nrm = sqrtf(s), inv = nrm > 0.f ? 1.f / nrm : 0.f;
     for (int i = lane; i < n; i += 32) V[(size_t)i * m + j] = ld(u + i) * inv;
-    if (lane == 0) W[j] = nrm - sigma;
+    if (lane == 0) W[j] = (nrm - sigma) * up;
   }
 }
 
