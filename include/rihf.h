@@ -245,7 +245,8 @@ int rihf_trace_stats(rihf_ctx* ctx, int max, char* names, double* launches, doub
    one n x n host matrix A (row-major, symmetric): eigenvalues W (n, ascending)
    and eigenvectors V (n x n, column k = eigenvector k).  FP32 parallel Jacobi
    (a cluster of CTAs) up to n = 256, tridiagonalisation in FP64 above, followed
-   by FP64 Ogita-Aishima refinement, on device `device`; n <= 4096.  Allocates
+   by FP64 Ogita-Aishima refinement, on device `device`; n <= 4096.  The norm of A
+   may lie anywhere from 1e-35 to 1e35 (above n = 256: 1e-140 to 1e140).  Allocates
    and frees its own device workspace.  Errors: INVALID_ARG, OOM, CUDA, TIMEOUT (a
    bounded device wait ran out). */
 int rihf_eigh(int n, const double* A, double* W, double* V, int device);
