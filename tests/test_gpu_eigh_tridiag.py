@@ -24,7 +24,16 @@ def _matrix(kind, n):
             A[k:k + m, k:k + m] = (B + B.T) / 2
         return A
     Q, _ = np.linalg.qr(rng.normal(size=(n, n)))
-    if kind == "graded":         # an overlap matrix of a nearly dependent basis
+    if kind == "rank 20":        # a null space of n - 20
+        w = np.where(np.arange(n) < 20, 1.0 + 0.05 * np.arange(n), 0.0)
+    elif kind == "projector":    # two eigenvalues, each n / 2 times, in an unreduced tridiagonal form
+        w = (np.arange(n) < n // 2).astype(float)
+    elif kind == "identity and noise":   # one cluster of all n, every coupling well above rounding
+        M = rng.normal(size=(n, n))
+        return np.eye(n) + 1e-13 * (M + M.T) / 2
+    elif kind == "decaying":     # from 1 down to far below rounding
+        w = np.logspace(-30, 0, n)
+    elif kind == "graded":         # an overlap matrix of a nearly dependent basis
         w = np.logspace(-9, 1, n)
     elif kind == "repeated":     # dense, a third of the eigenvalues equal
         w = np.where(np.arange(n) % 3 == 0, 1.0, np.linspace(-2, 2, n))
@@ -46,3 +55,23 @@ def test_special_spectra(kind, n):
     assert np.abs(W - ref).max() <= 1e-12 * scale
     assert np.abs(V.T @ V - np.eye(n)).max() <= 1e-12
     assert np.abs(A @ V - V * W).max() <= 1e-11 * scale
+
+
+@pytest.mark.parametrize("n", [257, 608])
+@pytest.mark.parametrize("kind", ["rank 20", "projector", "identity and noise", "decaying"])
+def test_large_clusters(kind, n):
+    """Eigenvalues close together in number: more than the 32 that one block orthogonalises, up to all
+    n.  Besides the bounds of the other spectra, the time: a generic matrix of order 608 takes 10 ms,
+    these at most that and four grid barriers a vector (2432, below 10 us each); orthogonalised on a
+    single SM they took 0.3 to 1.3 s."""
+    import time
+    from paper_2407_19614_gb300 import rihf as R
+    test_special_spectra(kind, n)
+    A = _matrix(kind, n)
+    A = (A + A.T) / 2
+    t = []
+    for _ in range(3):
+        t0 = time.perf_counter()
+        R.eigh(A)
+        t.append(time.perf_counter() - t0)
+    assert min(t) <= 0.05
