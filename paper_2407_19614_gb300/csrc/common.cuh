@@ -50,4 +50,18 @@ __host__ __device__ inline int cart_index(int l, int lx, int ly) {
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// Makes room for n elements in the array p of capacity cap, whose contents may go.
+// An allocation that throws leaves p empty with capacity zero, so that a later call
+// allocates again.
+template <class T, class Alloc, class Free>
+void regrow(T*& p, size_t& cap, size_t n, Alloc alloc, Free free) {
+  if (n <= cap) return;
+  T* old = p;
+  p = nullptr;
+  cap = 0;
+  if (old) free(old);
+  p = alloc(n);
+  cap = n;
+}
+
 }  // namespace rihf

@@ -732,13 +732,9 @@ static void refresh_tasks(rihf_ctx* c) {
     upload(c->d_tasks, list, c->stream);
     size_t n = 0;
     for (const auto& v : chunks) n += v.size();
-    if (n > c->chunk_cap) {
-      if (c->d_chunks) cudaFree(c->d_chunks);
-      c->d_chunks = nullptr;
-      c->lane = LaneTasks();
-      c->d_chunks = dalloc<LaneChunk>(n);
-      c->chunk_cap = n;
-    }
+    c->lane = LaneTasks();   // no launch from a list that is being replaced, should this throw
+    regrow(c->d_chunks, c->chunk_cap, n, [](size_t k) { return dalloc<LaneChunk>(k); },
+           [](LaneChunk* p) { cudaFree(p); });
     size_t at = 0;
     for (int g = 0; g < kLaneGroups; ++g) {
       c->lane.chunks[g] = c->d_chunks + at;
