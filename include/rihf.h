@@ -104,7 +104,7 @@ void rihf_default_options(rihf_options* opt);
  *   prim[nprim_shells], aux[naux_shells]: shells (atom indices into Z).
  *   nelec: electron count (even; closed shell).
  *   opt: options or NULL for the defaults.
- * Errors: INVALID_ARG (sizes, l limits, odd nelec), OOM, CUDA,
+ * Errors: INVALID_ARG (sizes, l limits, more than 4096 basis functions, odd nelec), OOM, CUDA, TIMEOUT,
  * NOT_POSITIVE_DEFINITE (metric or overlap).
  */
 int rihf_setup(int natoms, const int* Z, const double* xyz, int nprim_shells, const rihf_shell* prim,

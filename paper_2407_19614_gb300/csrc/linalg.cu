@@ -886,7 +886,7 @@ static void jacobi(const LaCtx& la, const double* A, int n, int m, float* gU, fl
 // Sort eigenpairs ascending (rank sort) and expand to FP64: X[:, rank] = V[:, i].
 __global__ void eig_sort_kernel(const float* __restrict__ V, const float* __restrict__ W, int n, int m, double* X,
                                 double* Wd) {
-  __shared__ int rank[4096];
+  __shared__ int rank[kEighMax];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     float wi = W[i];
     int r = 0;
@@ -1005,8 +1005,8 @@ static int elem_blocks(const LaCtx& la, long long n) {
 // FP64 pipe (257 us at n = 580 with them, every block ranking all values).
 __global__ void eig_sort64_kernel(const double* __restrict__ V, const double* __restrict__ lam, int n, double* Vout,
                                   double* Wout) {
-  __shared__ unsigned long long key[4096];
-  __shared__ int rank[4096];
+  __shared__ unsigned long long key[kEighMax];
+  __shared__ int rank[kEighMax];
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(lam[i] + 0.0);   // -0 as +0
     key[i] = b >> 63 ? ~b : b | 1ull << 63;
@@ -1028,6 +1028,7 @@ __global__ void eig_sort64_kernel(const double* __restrict__ V, const double* __
 
 void eigh(const LaCtx& la, const double* A, int n, double* W, double* V, double* ws, int refine,
           const double* Vguess, bool skip_jacobi, int max_sweeps, int ns_steps) {
+  if (n > kEighMax) throw RihfError(RIHF_ERR_INVALID_ARG, "eigensolver: order above its limit");
   int m = n + (n & 1);
   if (skip_jacobi && Vguess && refine > 0) {
     // Late SCF iterations: the previous eigenvectors are already close, so the

@@ -98,6 +98,7 @@ void trsm_lower(const LaCtx& la, const double* L, int n, double* X, long long nc
 // even order m), then six n x n FP64 refinement matrices and 2n + 8 scalars;
 // above kJacobiMax also tridiag_workspace(n).
 constexpr int kJacobiMax = 256;
+constexpr int kEighMax = 4096;   // largest order: ranks and cluster marks are in shared memory
 constexpr int kTridiagRefine = 2;
 constexpr size_t eig_workspace_base(int n) {
   return ((size_t)(n + (n & 1)) * (n + (n & 1)) + (size_t)n * (n + (n & 1)) + (n + (n & 1)) + 1) / 2 +

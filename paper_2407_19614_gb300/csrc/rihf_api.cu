@@ -1345,6 +1345,16 @@ int rihf_setup(int natoms, const int* Z, const double* xyz, int nprim_shells, co
     return RIHF_ERR_INVALID_ARG;
   }
   *out = nullptr;
+  {   // the eigensolver's sorting and cluster kernels hold one entry an eigenvalue in shared memory
+    const bool pure = !opt || opt->pure != 0;
+    long long N = 0;
+    for (int i = 0; i < nprim_shells; ++i)
+      if (prim[i].l >= 0 && prim[i].l <= kMaxLPrim) N += pure ? nsph(prim[i].l) : ncart(prim[i].l);
+    if (N > kEighMax) {
+      g_last_error = "more than " + std::to_string(kEighMax) + " basis functions";
+      return RIHF_ERR_INVALID_ARG;
+    }
+  }
   *out = setup_impl(natoms, Z, xyz, nprim_shells, prim, naux_shells, aux, nelec, opt, nullptr);
   return RIHF_OK;
   RIHF_API_END
@@ -3257,7 +3267,7 @@ int rihf_trace_stats(rihf_ctx* c, int max, char* names, double* launches, double
 
 int rihf_eigh(int n, const double* A, double* W, double* V, int device) {
   RIHF_API_BEGIN
-  if (n <= 0 || n > 4096 || !A || !W || !V) return RIHF_ERR_INVALID_ARG;
+  if (n <= 0 || n > kEighMax || !A || !W || !V) return RIHF_ERR_INVALID_ARG;
   RIHF_CUDA(cudaSetDevice(device));
   cudaStream_t s;
   RIHF_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));

@@ -109,3 +109,24 @@ def test_no_cpu_fallback_without_a_device(libpath):
     R.load(libpath)
     with pytest.raises(R.RihfError, match="CUDA"):
         R.Context(W.water_monomer(0))
+
+
+def test_basis_beyond_the_eigensolver_is_refused(libpath):
+    """4097 functions: the eigensolver's shared-memory tables end at 4096.  Refused before any device
+    call (shells of one s function each; with 4096 the call goes on and fails for want of a device)."""
+    import types
+    import numpy as np
+    import torch
+    from paper_2407_19614_gb300 import rihf as R
+    from paper_2407_19614_gb300 import workloads as W
+    R.load(libpath)
+
+    def mol(n):
+        return types.SimpleNamespace(Z=np.array([2]), xyz=np.zeros((1, 3)), primary=[W.Shell(0, 0, [1.0], [1.0])] * n,
+                                     aux=[W.Shell(0, 0, [1.0], [1.0])])
+
+    with pytest.raises(R.RihfError, match="4096 basis functions"):
+        R.Context(mol(4097))
+    if not torch.cuda.is_available():
+        with pytest.raises(R.RihfError, match="CUDA"):
+            R.Context(mol(4096))
