@@ -1,17 +1,17 @@
 // Derivative contraction of the one-electron integrals for spherical bases:
-// kOneLanes lanes per shell pair, which share out the nuclei and, for overlap and
-// kinetic energy, the Cartesian components.
+// 4 to 32 lanes per shell pair (build_one_tasks), which share out the nuclei and, for
+// overlap and kinetic energy, the Cartesian components.
 //
 // The derivative of nuclear attraction needs the weights w of the horizontal
 // recurrence applied to D (grad_lane.cuh) once per pair; each nucleus then costs
 // its recursion and one pass of dot products, its own force being minus the
 // translation 2p U - D + 2 beta AB V of the pair.  (A, B) terms are linear in the
 // integrals and are contracted once, from the sum over nuclei.
-// Bound by FP64 instructions, at small sizes by the latency of one pair.  0.27 ms at
-// (H2O)8 (4656 pairs, 24 nuclei), 1.07 ms at (H2O)10 in the larger basis; the
+// Bound by FP64 instructions, at small sizes by the latency of one pair.  0.086 ms at
+// (H2O)3 (666 pairs, 9 nuclei), 0.137 at (H2O)8, 1.08 at (H2O)10 in the larger basis; the
 // warp-cooperative kernel (a task per pair and nucleus, four recurrences each) takes
-// 0.95 and 16.4 ms.  At (H2O)3 it is the slower one, 0.18 against 0.11 ms: a (d d|
-// pair's serial chain; one kernel for all sizes was preferred.
+// 0.105, 0.95 and 16.4 ms.  One water in the larger basis is the one case where it is
+// ahead, 0.182 against 0.199 ms: the serial chain of an (f f| pair.
 #include <algorithm>
 
 #include "../../include/rihf.h"
@@ -34,8 +34,9 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
   constexpr int E = LA + LB + 1, EMIN = LA > 0 ? LA - 1 : 0, O = cart_offset(EMIN), NK = cart_offset(E + 1) - O;
   constexpr int NA = ncart(LA), NB = ncart(LB), OW = cart_offset(LA), NW = cart_offset(LA + LB + 1) - OW, LD = LB + 3;
   constexpr int kUnroll = LA + LB < 6 ? 64 : 1;   // (f f|: rolled, for the compiler's sake
-  const int lane = threadIdx.x, q = lane % kOneLanes, j = min(lane / kOneLanes, ch.n - 1);
-  const bool live = lane / kOneLanes < ch.n;
+  const int L = g.lanes, lane = threadIdx.x, q = lane & (L - 1), slot = lane >> (31 - __clz(L));
+  const int j = min(slot, ch.n - 1);
+  const bool live = slot < ch.n;
   const DevShells& pr = g.prim;
   const int2 tk = g.tasks[ch.task0 + j];
   const int sa = tk.x, sb = tk.y, N = pr.nfunc, ta = pr.atom[sa], tb = pr.atom[sb];
@@ -65,7 +66,7 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
         overlap_1d<LA + 1, LB + 2, LD>(d.PA[x], d.PA[x] + AB[x], 0.5 * d.ip, x == 0 ? cc * d.K : 1.0, s[x]);
       const double f = 3.14159265358979323846 * d.ip, f3 = f * sqrt(f);
 #pragma unroll 1
-      for (int at = q; at < NA * NB; at += kOneLanes) {   // the lanes share out the components
+      for (int at = q; at < NA * NB; at += L) {   // the lanes share out the components
         int c[3], e[3];
         cart_decode(LA, at / NB, c[0], c[1], c[2]);
         cart_decode(LB, at % NB, e[0], e[1], e[2]);
@@ -99,7 +100,7 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
     for (int i = 0; i < NK; ++i) ks[i] = 0.0;
     const double pref = -6.283185307179586 * d.ip * cc * d.K;
 #pragma unroll 1
-    for (int c0 = 0; c0 < g.natoms; c0 += kOneLanes) {
+    for (int c0 = 0; c0 < g.natoms; c0 += L) {
       const int c = min(c0 + q, g.natoms - 1);
       const double z = c0 + q < g.natoms ? (double)g.Z[c] : 0.0;
       const double CP[3] = {g.axyz[3 * c] - d.P[0], g.axyz[3 * c + 1] - d.P[1], g.axyz[3 * c + 2] - d.P[2]};
@@ -129,9 +130,9 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         double t = -fma(2.0 * be * AB[i], V, U[i]);
-#pragma unroll
-        for (int o = kOneLanes; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane < kOneLanes && c0 + q < g.natoms) atomicAdd(grad_one + 3 * c + i, t);
+#pragma unroll 1
+        for (int o = L; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane < L && c0 + q < g.natoms) atomicAdd(grad_one + 3 * c + i, t);
       }
     }
     double s[10];
@@ -145,10 +146,10 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
       gB[x] += fma(2.0 * be, fma(AB[x], s[9], s[x]), -s[6 + x]);
     }
   }
+#pragma unroll 1
+  for (int o = L / 2; o > 0; o >>= 1)
 #pragma unroll
-  for (int x = 0; x < 3; ++x)
-#pragma unroll
-    for (int o = kOneLanes / 2; o > 0; o >>= 1) {
+    for (int x = 0; x < 3; ++x) {
       gA[x] += __shfl_xor_sync(0xffffffffu, gA[x], o);
       gB[x] += __shfl_xor_sync(0xffffffffu, gB[x], o);
       gS[x] += __shfl_xor_sync(0xffffffffu, gS[x], o);

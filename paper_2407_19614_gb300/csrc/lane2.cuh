@@ -10,6 +10,7 @@ struct Lane2Tasks {
   const int2* tasks = nullptr;
   const LaneChunk* chunks = nullptr;
   long long nchunk = 0;
+  int lanes = 1;   // lanes a task
 };
 
 // (P|Q): auxiliary shell pairs, the lower l first; cls = la | lc << 8.
@@ -21,10 +22,9 @@ void launch_lane_eri2(const IntegralCtx& ic, const DevShells& aux, const Lane2Ta
 void launch_lane_grad_eri2(const IntegralCtx& ic, const DevShells& aux, const Lane2Tasks& t, const KetTable* ket,
                            const double* Z, double* grad);
 
-// One-electron: primary shell pairs (a, b), la >= lb, kOneLanes lanes each (the
-// nuclei shared out between them); cls = la | lb << 4.
-constexpr int kOneLanes = 4;
-void build_one_tasks(const std::vector<int>& l, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks);
+// One-electron: primary shell pairs (a, b), la >= lb, 4 to 32 lanes each (the
+// nuclei shared out between them), the number returned; cls = la | lb << 4.
+int build_one_tasks(const std::vector<int>& l, int sms, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks);
 // S and h = T + V, both triangles.
 void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
                      const double* axyz, double* S, double* H);

@@ -1,9 +1,8 @@
-// One-electron integrals for spherical bases: kOneLanes lanes per shell pair, which
+// One-electron integrals for spherical bases: 4 to 32 lanes per shell pair, which
 // share out the nuclei (the recursion of eri3_lane.cuh with a point-charge ket, i.e.
-// no ket steps).  Four lanes a pair: one warp per SM sub-partition at (H2O)8, where the
-// latency of one pair is the time; more lanes repeat the per-pair part more often.
-// Measured 0.10 ms at (H2O)8 (4656 pairs, 24 nuclei), 0.38 ms at (H2O)10 in the larger
-// basis; the warp-cooperative kernel takes 0.40 and 3.1 ms.
+// no ket steps; how many lanes: build_one_tasks).  Measured 0.077 ms at (H2O)8 (4656
+// pairs, 24 nuclei), 0.38 ms at (H2O)10 in the larger basis; the warp-cooperative
+// kernel takes 0.39 and 3.1 ms.
 #include <algorithm>
 
 #include "../../include/rihf.h"
@@ -17,7 +16,8 @@ template <int LA, int LB>
 __device__ __noinline__ void one_tasks(const OneArgs& g, const LaneChunk& ch, double* __restrict__ S, double* __restrict__ H) {
   constexpr int E = LA + LB, O = cart_offset(LA), NK = cart_offset(E + 1) - O;
   constexpr int NA = ncart(LA), NB = ncart(LB), FA = nsph(LA), FB = nsph(LB), LD = LB + 3;
-  const int q = threadIdx.x % kOneLanes, j = min((int)threadIdx.x / kOneLanes, ch.n - 1);   // idle lanes repeat the last
+  const int L = g.lanes, q = threadIdx.x & (L - 1), slot = threadIdx.x >> (31 - __clz(L));
+  const int j = min(slot, ch.n - 1);   // idle lanes repeat the last
   const DevShells& pr = g.prim;
   const int2 tk = g.tasks[ch.task0 + j];
   const int sa = tk.x, sb = tk.y, N = pr.nfunc;
@@ -67,7 +67,7 @@ __device__ __noinline__ void one_tasks(const OneArgs& g, const LaneChunk& ch, do
             }
       const double pref = 6.283185307179586 * d.ip * w * d.K;
 #pragma unroll 1
-      for (int c = q; c < g.natoms; c += kOneLanes) {
+      for (int c = q; c < g.natoms; c += L) {
         const double CP[3] = {g.axyz[3 * c] - d.P[0], g.axyz[3 * c + 1] - d.P[1], g.axyz[3 * c + 2] - d.P[2]};
         double F[E + 1], row[cart_offset(E + 1)];
         lane_boys<E>(0, d.p * fma(CP[0], CP[0], fma(CP[1], CP[1], CP[2] * CP[2])), g.boys, F);
@@ -76,11 +76,11 @@ __device__ __noinline__ void one_tasks(const OneArgs& g, const LaneChunk& ch, do
         for (int e = 0; e < NK; ++e) k[e] += row[O + e];
       }
     }
+#pragma unroll 1
+  for (int o = L / 2; o > 0; o >>= 1)
 #pragma unroll
-  for (int e = 0; e < NK; ++e)
-#pragma unroll
-    for (int o = kOneLanes / 2; o > 0; o >>= 1) k[e] += __shfl_xor_sync(0xffffffffu, k[e], o);
-  if (q != 0 || (int)threadIdx.x / kOneLanes >= ch.n) return;
+    for (int e = 0; e < NK; ++e) k[e] += __shfl_xor_sync(0xffffffffu, k[e], o);
+  if (q != 0 || slot >= ch.n) return;
   double v[NA * NB], out[FA * FB];
   lane_hrr<LA, LB>(k, AB, v);
 #pragma unroll
@@ -108,7 +108,16 @@ __global__ void __launch_bounds__(32, 8) lane_one_kernel(const __grid_constant__
 }
 }  // namespace
 
-void build_one_tasks(const std::vector<int>& l, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks) {
+// The lanes of a pair: the most that leave at most 32 warps an SM.  Below that the
+// latency of one pair's chain over the nuclei is the time, and more lanes shorten it;
+// above, FP64 instructions count and the part of a pair that every lane repeats makes
+// more lanes dearer.  Derivatives with 4 / 8 / 16 / 32 lanes: (H2O)3, 666 pairs, 0.176 /
+// 0.135 / 0.100 / 0.084 ms; (H2O)8, 4656 pairs, 0.268 / 0.176 / 0.143 / 0.139; (H2O)12,
+// 10440 pairs, 0.397 / 0.276 / 0.272 / 0.387.
+int build_one_tasks(const std::vector<int>& l, int sms, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks) {
+  const long long pairs = (long long)l.size() * (l.size() + 1) / 2;
+  int lanes = 32;
+  while (lanes > 4 && pairs * lanes > 32LL * 32 * sms) lanes /= 2;
   std::vector<int> by_l[kMaxLPrim + 1];
   for (int i = 0; i < (int)l.size(); ++i) by_l[l[i]].push_back(i);
   tasks.clear();
@@ -120,9 +129,10 @@ void build_one_tasks(const std::vector<int>& l, std::vector<int2>& tasks, std::v
         for (int b : by_l[lb])
           if (la != lb || a >= b) tasks.push_back(make_int2(a, b));
       const long long n = (long long)tasks.size() - t0;
-      constexpr int per = 32 / kOneLanes;
+      const int per = 32 / lanes;
       for (long long i = 0; i < n; i += per) chunks.push_back({t0 + i, (int)std::min<long long>(per, n - i), la | lb << 4});
     }
+  return lanes;
 }
 
 void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,

@@ -83,6 +83,7 @@ struct OneArgs {
   DevShells prim;
   const int2* tasks;
   const LaneChunk* chunks;
+  int lanes;      // per pair: 4, 8, 16 or 32
   int natoms;
   const int* Z;
   const double* axyz;
@@ -91,7 +92,7 @@ struct OneArgs {
 
 inline OneArgs one_args(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
                         const double* axyz) {
-  return OneArgs{prim, t.tasks, t.chunks, natoms, Z, axyz, ic.boys};
+  return OneArgs{prim, t.tasks, t.chunks, t.lanes, natoms, Z, axyz, ic.boys};
 }
 
 // Runs f<la, lb>(g, ch, ...) for the class of chunk ch.

@@ -1197,7 +1197,7 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       std::vector<int2> t2, t1;
       std::vector<LaneChunk> c2, c1;
       build_lane2_tasks(c->ha.l, c->ha.atom, t2, c2);
-      build_one_tasks(c->hp.l, t1, c1);
+      const int lanes = build_one_tasks(c->hp.l, c->sms, t1, c1);
       c->d_tasks2 = dalloc<int2>(t2.size() + t1.size());
       c->d_chunks2 = dalloc<LaneChunk>(c2.size() + c1.size());
       upload(c->d_tasks2, t2, s);
@@ -1206,7 +1206,7 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       upload(c->d_chunks2 + c2.size(), c1, s);
       RIHF_CUDA(cudaStreamSynchronize(s));   // the host lists are temporaries
       c->lane_eri2 = {c->d_tasks2, c->d_chunks2, (long long)c2.size()};
-      c->lane_one = {c->d_tasks2 + t2.size(), c->d_chunks2 + c2.size(), (long long)c1.size()};
+      c->lane_one = {c->d_tasks2 + t2.size(), c->d_chunks2 + c2.size(), (long long)c1.size(), lanes};
     }
     refresh_tasks(c);
     {
