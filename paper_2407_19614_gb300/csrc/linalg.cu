@@ -7,6 +7,7 @@
 
 #include "../../include/rihf.h"
 #include "eigh_tridiag.cuh"
+#include "gemm_index.cuh"
 #include "linalg.cuh"
 #include "tc_gemm.cuh"
 
@@ -38,21 +39,6 @@ static inline void count(const LaCtx& la, int n = 1) {
 
 // ------------------------------------------------------------ GEMM (FP64)
 
-// C tiles of 16 x 16 by 128-thread CTAs, two elements a thread.  FP64 bounds every
-// product here (two FMAs per clock and SM), so what counts is that no tile is
-// mostly padding and that the tiles fill the SMs evenly: 16 is the largest tile
-// that gives a 192 x 192 result one CTA per SM (144) without splitting K, and wastes
-// least at the 40 columns of H = B C~ (48 computed; 64 with a 32-wide tile).  The
-// operands come through a ring of three K chunks filled by cp.async two chunks
-// ahead.  Measured, 192 x 192 x 192: 18 us, 14 us for a symmetric result, against
-// 17 us plus a 5 us reduction of split sums with 32 x 32 tiles; H and K of an FP64
-// Fock build at N = 192, Naux = 848 (40 occupied): 3.6 ms against 5.7.
-constexpr int GT = 16;        // output tile
-constexpr int GK = 32;        // K chunk, at most
-constexpr int GS = 3;         // chunks in flight
-constexpr int GThreads = 128;
-constexpr int kGemmCluster = 8;   // most K slices summed through a thread-block cluster
-
 // Eight-byte asynchronous copy; zero when the element does not exist.
 __device__ __forceinline__ void gemm_cp8(double* dst, const double* src, bool valid) {
   const unsigned at = (unsigned)__cvta_generic_to_shared(dst);
@@ -64,20 +50,6 @@ __device__ __forceinline__ void gemm_store(const GemmArgs& g, double* C, int m, 
   if (m >= g.M || n >= g.N) return;
   double* c = C + (long long)m * g.ldc + n;
   *c = g.beta == 0.0 ? g.alpha * v : g.alpha * v + g.beta * *c;
-}
-
-// Tile t of the result: all tiles row by row, or (lower_only) those on and below
-// the diagonal.
-__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int t, int tn, int& tm, int& tc) {
-  if (!g.lower_only) {
-    tm = t / tn;
-    tc = t - tm * tn;
-    return;
-  }
-  tm = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
-  while (tm * (tm + 1) / 2 > t) --tm;
-  while ((tm + 1) * (tm + 2) / 2 <= t) ++tm;
-  tc = t - tm * (tm + 1) / 2;
 }
 
 // grid.x: tiles x batches; grid.y: slices of the sum (K, or the batches when they
@@ -92,20 +64,9 @@ __global__ void __launch_bounds__(GThreads) dgemm_kernel(GemmArgs g, int tiles, 
   __shared__ double As[GS][GK][GT + 1], Bs[GS][GK][GT + 1];
   __shared__ double part[GT * GT];
   const int tid = threadIdx.x;
-  const int batch = blockIdx.x / tiles, slice = blockIdx.y;
-  int tm, tc;
-  gemm_tile(g, blockIdx.x - batch * tiles, tn, tm, tc);
-  const int m0 = tm * GT, n0 = tc * GT;
-  int b0 = batch, b1 = batch + 1, k0 = 0, k1 = g.K;
-  if (g.reduce_batch) {
-    b0 = slice * bper;
-    b1 = min(g.batch, b0 + bper);
-  } else {
-    k0 = slice * kper;
-    k1 = min(g.K, k0 + kper);
-  }
-  const int per = k1 > k0 ? (k1 - k0 + chunk - 1) / chunk : 0;   // chunks of one batch
-  const int total = b1 > b0 ? (b1 - b0) * per : 0;
+  const GemmBlock q = gemm_block(g, blockIdx.x, blockIdx.y, tiles, tn, kper, bper, chunk);
+  const int batch = q.batch, slice = blockIdx.y, m0 = q.m0, n0 = q.n0, b0 = q.b0, k0 = q.k0, k1 = q.k1, per = q.per,
+            total = q.total;
   auto fetch = [&](int c) {
     if (c < total) {
       const int b = b0 + c / per, kc = k0 + (c % per) * chunk;
@@ -113,13 +74,9 @@ __global__ void __launch_bounds__(GThreads) dgemm_kernel(GemmArgs g, int tiles, 
       const double* B = g.B + (long long)b * g.sB;
       const int st = c % GS;
       for (int idx = tid; idx < GT * chunk; idx += GThreads) {
-        int mm, ka, nn, kb;
-        if (TA) { mm = idx % GT; ka = idx / GT; } else { ka = idx % chunk; mm = idx / chunk; }
-        if (TB) { kb = idx % chunk; nn = idx / chunk; } else { nn = idx % GT; kb = idx / GT; }
-        const int m = m0 + mm, n = n0 + nn, x = kc + ka, y = kc + kb;
-        const bool va = m < g.M && x < k1, vb = n < g.N && y < k1;
-        gemm_cp8(&As[st][ka][mm], va ? (TA ? A + (long long)x * g.lda + m : A + (long long)m * g.lda + x) : A, va);
-        gemm_cp8(&Bs[st][kb][nn], vb ? (TB ? B + (long long)n * g.ldb + y : B + (long long)y * g.ldb + n) : B, vb);
+        const GemmElem a = gemm_elem<!TA>(idx, chunk, m0, g.M, kc, k1, g.lda), b = gemm_elem<TB>(idx, chunk, n0, g.N, kc, k1, g.ldb);
+        gemm_cp8(&As[st][a.k][a.row], A + a.at, a.valid);
+        gemm_cp8(&Bs[st][b.k][b.row], B + b.at, b.valid);
       }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -220,58 +177,22 @@ void dgemm(const LaCtx& la, const GemmArgs& g) {
     if (g.mirror) symmetrize_lower(la, g.C, g.N, 1);
     return;
   }
-  const int tm = ceil_div(g.M, GT), tn = ceil_div(g.N, GT);
-  const int nb = g.reduce_batch ? 1 : g.batch;
-  if ((long long)tm * tn > 0x7fffffffLL / nb)
-    throw RihfError(RIHF_ERR_INVALID_ARG, "dgemm: too many tiles for this product shape");
-  const int tiles = g.lower_only ? tm * (tm + 1) / 2 : tm * tn;
-  // the chunk divides K when K is short (reduced batches of K = nocc: no padded steps)
-  const int chunk = std::max(1, ceil_div(g.K, ceil_div(std::max(1, g.K), GK)));
-  // Slices: the least time of the fullest SM, in FP64 steps of one tile: a CTA alone
-  // on its SM takes 1.75 times its FP64 time (one warp per sub-partition: 226 clocks
-  // a step instead of 128, measured at 192 x 192 x 192), so two half slices beat one
-  // whole; and a slice costs some steps beside its own (filling the ring, the sum).
-  // Up to kGemmCluster slices are summed in a cluster; more go through la.work, which
-  // has to hold them, and only where a long reduction leaves each slice long.
-  const long long ctas = (long long)tiles * nb;
-  const long long len = g.reduce_batch ? (long long)g.batch * g.K : g.K;
-  const long long most_len = g.reduce_batch ? g.batch : std::max(1, g.K / 8);   // at least 8 of K a slice
-  int nslice = 1;
-  double best = 1e300;
-  for (int s = 1; s <= 64 && s <= most_len; ++s) {
-    if (s > kGemmCluster &&
-        ((size_t)s * g.M * g.N * nb > la.work_elems || len / s < 512)) break;
-    const double steps = (double)ceil_div(len, s) + (s > 1 ? 16.0 : 8.0) + (s > kGemmCluster ? 40.0 : 0.0);
-    const double cost = std::max((double)((ctas * s + la.sms - 1) / la.sms), 1.75) * steps;
-    if (cost < 0.98 * best) {
-      best = cost;
-      nslice = s;
-    }
-  }
-  int kper = g.K, bper = g.batch;
-  if (g.reduce_batch) {
-    bper = ceil_div(g.batch, nslice);
-    nslice = ceil_div(g.batch, bper);
-  } else if (nslice > 1) {
-    kper = ceil_div(g.K, nslice);
-    nslice = ceil_div(g.K, kper);
-  }
-  const int cluster = nslice > 1 && nslice <= kGemmCluster ? 1 : 0;
+  const GemmPlan p = gemm_plan(g, la.sms, la.work_elems);
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr{};
-  cfg.gridDim = dim3((unsigned)ctas, (unsigned)nslice, 1);
+  cfg.gridDim = dim3((unsigned)p.ctas, (unsigned)p.nslice, 1);
   cfg.blockDim = dim3(GThreads, 1, 1);
   cfg.stream = la.stream;
-  if (cluster) {
+  if (p.cluster) {
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = 1;
-    attr.val.clusterDim.y = (unsigned)nslice;
+    attr.val.clusterDim.y = (unsigned)p.nslice;
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
   }
   auto run = [&](auto kernel) {
-    RIHF_CUDA(cudaLaunchKernelEx(&cfg, kernel, g, tiles, tn, nslice, kper, bper, chunk, cluster, la.work));
+    RIHF_CUDA(cudaLaunchKernelEx(&cfg, kernel, g, p.tiles, p.tn, p.nslice, p.kper, p.bper, p.chunk, p.cluster, la.work));
   };
   auto pick = [&](auto full) {
     constexpr bool F = decltype(full)::value;
@@ -280,13 +201,13 @@ void dgemm(const LaCtx& la, const GemmArgs& g) {
     else if (g.transB) run(dgemm_kernel<false, true, F>);
     else run(dgemm_kernel<false, false, F>);
   };
-  if (chunk == GK) pick(std::true_type());
+  if (p.chunk == GK) pick(std::true_type());
   else pick(std::false_type());
   count(la);
-  if (nslice > 1 && !cluster) {
-    const long long total = (long long)g.M * g.N * nb;
+  if (p.nslice > 1 && !p.cluster) {
+    const long long total = (long long)g.M * g.N * (g.reduce_batch ? 1 : g.batch);
     const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * la.sms);
-    splitk_reduce_kernel<<<blocks, 256, 0, la.stream>>>(g, nslice, la.work);
+    splitk_reduce_kernel<<<blocks, 256, 0, la.stream>>>(g, p.nslice, la.work);
     RIHF_LAUNCH_CHECK();
     count(la);
   }
