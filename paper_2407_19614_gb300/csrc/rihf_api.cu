@@ -629,7 +629,7 @@ struct rihf_ctx {
   double* trsm_tmp = nullptr;
   double *cvec = nullptr, *W = nullptr, *Bij = nullptr, *Xt = nullptr, *Zm = nullptr;
   double* G = nullptr;   // the gradient's G' = C~ X~ (shares Hb's memory: H is spent by then)
-  double* grad_parts = nullptr;   // 5 x natoms x 3 on device (one, overlap, three, two, nuc)
+  double* grad_parts = nullptr;   // 4 x natoms x 3 (one, overlap, three, two), then d_flag's four ints
   std::vector<double> grad_parts_h;
 
   double* work = nullptr;
@@ -777,7 +777,7 @@ static void free_all(rihf_ctx* c) {
                   c->d_ao_atom, c->d_ao_l, c->hist_D[0], c->hist_D[1], c->hist_D[2], c->hist_S, c->hist_xyz[0],
                   c->hist_xyz[1], c->Shalf, c->Smhalf, c->DL, c->Dpred, c->mlX, c->mly, c->mlt, c->mlDx, c->ml_sums, c->rep_X, c->rep_t, c->net.master, c->net.wbf, c->net.grad,
                   c->net.m, c->net.v, c->net.loss,
-                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_flag, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_chunks, c->d_ket, c->d_tasks2, c->d_chunks2, c->d_schwarz,
+                  c->d_tr, c->d_nf, c->d_Z, c->d_xyz, c->d_boys, c->d_counter, c->d_sched, c->d_red, c->d_ticket, c->d_pairs, c->d_tasks, c->d_chunks, c->d_ket, c->d_tasks2, c->d_chunks2, c->d_schwarz,
                   c->S, c->H, c->Tk, c->V, c->A, c->L, c->Linv, c->Bp, c->Yp, c->Bu, c->Dp, c->Jp, c->Xo, c->Sw, c->Sv,
                   c->C, c->eps, c->Ct, c->D, c->J, c->K, c->F, c->Fx, c->T1, c->T2, c->Err, c->Fp, c->Cp, c->Hb,
                   c->dvec, c->Fring, c->Ering, c->Bdiis, c->coef, c->scal, c->Cprev,
@@ -1045,7 +1045,8 @@ static void compute_geometry_rest(rihf_ctx* c) {
     RIHF_CUDA(cudaMemcpyAsync(c->Xo, c->T1, sizeof(double) * N * nind, cudaMemcpyDeviceToDevice, s));
   }
   cudaEventRecord(c->ev[1], s);
-  RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
+  if (c->tcA.planes)   // the products since the last look wait on the device only on the tensor cores
+    RIHF_CUDA(cudaMemcpyAsync(flag, c->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
   RIHF_CUDA(cudaStreamSynchronize(s));
   if (flag[1]) late();
   c->tracer.flush();
@@ -1171,7 +1172,6 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
     c->d_xyz = dalloc<double>(3 * natoms);
     c->d_boys = dalloc<double>((size_t)kBoysN * kBoysM); upload(c->d_boys, boys_host(), s);
     c->d_counter = dalloc<int>(4);
-    c->d_flag = dalloc<int>(4);
     c->d_sched = dalloc<int>(2);
     RIHF_CUDA(cudaMemset(c->d_sched, 0, 2 * sizeof(int)));
     c->d_red = dalloc<double>(kRedSlots);
@@ -1279,7 +1279,8 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       c->rep_X = dalloc<float>(M * kMlpF * rihf_ctx::kReplay);
       c->rep_t = dalloc<float>(M * rihf_ctx::kReplay);
     }
-    c->grad_parts = dalloc<double>(5 * 3 * natoms);
+    c->grad_parts = dalloc<double>(4 * 3 * natoms + 2);   // the error words after the parts: one copy brings both
+    c->d_flag = reinterpret_cast<int*>(c->grad_parts + 12 * natoms);
     c->work_elems = std::max<size_t>({(size_t)1 << 24, 8 * n2 * 4, (size_t)NA * 64});
     c->work = dalloc<double>(c->work_elems);
     c->eigws = dalloc<double>(eig_workspace(N));
@@ -2698,7 +2699,7 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
     }
   }
   // fused derivative-integral contractions
-  RIHF_CUDA(cudaMemsetAsync(c->grad_parts, 0, sizeof(double) * 15 * nat, s));
+  RIHF_CUDA(cudaMemsetAsync(c->grad_parts, 0, sizeof(double) * 12 * nat, s));
   double* g_one = c->grad_parts;
   double* g_ovl = c->grad_parts + 3 * nat;
   double* g_three = c->grad_parts + 6 * nat;
@@ -2724,14 +2725,15 @@ static void gradient_finish(rihf_ctx* c, double* grad) {
   cudaStream_t s = c->stream;
   const int nat = c->natoms;
   c->grad_parts_h.assign(15 * nat, 0.0);
-  RIHF_CUDA(cudaMemcpyAsync(c->grad_parts_h.data(), c->grad_parts, sizeof(double) * 12 * nat,
+  RIHF_CUDA(cudaMemcpyAsync(c->grad_parts_h.data(), c->grad_parts, sizeof(double) * (12 * nat + 2),
                             cudaMemcpyDeviceToHost, s));
-  int late = 0;
-  RIHF_CUDA(cudaMemcpyAsync(&late, c->d_flag + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
   cudaEventRecord(c->ev[6], s);
   RIHF_CUDA(cudaStreamSynchronize(s));
   c->tracer.flush();
-  if (late) {
+  int flag[4];
+  std::memcpy(flag, c->grad_parts_h.data() + 12 * nat, sizeof(flag));
+  std::fill_n(c->grad_parts_h.begin() + 12 * nat, 2, 0.0);
+  if (flag[1]) {
     late_clear(c);
     throw RihfError(RIHF_ERR_TIMEOUT, "gradient: a bounded device wait ran out");
   }
