@@ -924,6 +924,12 @@ static void compute_geometry(rihf_ctx* c, bool defer_eri3 = false) {
   compute_geometry_rest(c);
 }
 
+// BF16 MMA operations of a triangular solve with digit-plane updates: every digit pair
+// of the products outside the FP64 panels of kTrsmPanel rows.
+static double trsm_tc_flops(int n, long long ncol) {
+  return (double)n * std::max(0, n - kTrsmPanel) * ncol * oz_products(kOzMaxDigits);
+}
+
 // The fit, the planes or expansion of B and the orthogonaliser, after the
 // 3-centre integrals of this geometry are in Bp.
 static void compute_geometry_rest(rihf_ctx* c) {
@@ -932,7 +938,7 @@ static void compute_geometry_rest(rihf_ctx* c) {
   LaCtx la = c->la();
   if (c->trsm_sc.X.planes) {
     // mixed mode: rank-64 updates on the tensor cores (7 digits), panels in FP64
-    TraceScope t(c->tracer, s, "fit trsm B=L^-1 T (tcgen05 digit updates)", (double)NA * NA * c->npp, 0);
+    TraceScope t(c->tracer, s, "fit trsm B=L^-1 T (tcgen05 digit updates)", trsm_tc_flops(NA, c->npp), 3);
     trsm_lower_tc(la, c->L, NA, c->Bp, c->npp, 0, c->trsm_sc);
   } else {
     TraceScope t(c->tracer, s, "fit trsm B=L^-1 T", (double)NA * NA * c->npp, 0);
@@ -1631,7 +1637,7 @@ static void fock_build(rihf_ctx* c) {
   gk.B = c->Hb; gk.ldb = no; gk.sB = (long long)N * no; gk.transB = true;
   gk.C = c->K; gk.ldc = N; gk.batch = NA; gk.reduce_batch = true; gk.alpha = -0.5;
   gk.lower_only = gk.mirror = true;   // K is symmetric
-  { TraceScope t(c->tracer, c->stream, "RI-K K=-1/2 sum H H^T (dgemm)", 2.0 * NA * n2 * no, 0);
+  { TraceScope t(c->tracer, c->stream, "RI-K K=-1/2 sum H H^T (dgemm)", (double)NA * N * (N + 1) * no, 0);   // lower triangle
     dgemm(la, gk); }
   add3(la, (int)n2, c->H, c->J, c->K, c->F);
   if (c->sph_avg) {
@@ -2608,11 +2614,12 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   }
   // [X~ | c] = L^{-T} [Bij | d]  (NA x (nocc^2 + 1)): the paper's X^P_ij = sum_Q A^L_PQ B^Q_ij
   // and L^P in one blocked solve (the solve is latency-bound, one extra column is free)
+  const bool trsm_tc = c->trsm_sc.X.planes && oz_plane_elems(ldx, kTrsmOuter, kOzMaxDigits) <= c->trsm_sc.X.cap;
   { TraceScope t(c->tracer, s, "grad [X | c] = L^-T [Bij | d] (trsm; tcgen05 updates in mixed mode)",
-                 (double)NA * NA * ldx, 0);
+                 trsm_tc ? trsm_tc_flops(NA, ldx) : (double)NA * NA * ldx, trsm_tc ? 3 : 0);
     RIHF_CUDA(cudaMemcpy2DAsync(c->Xt + (size_t)no * no, ldx * sizeof(double), c->dvec, sizeof(double),
                                 sizeof(double), NA, cudaMemcpyDeviceToDevice, s));
-    if (c->trsm_sc.X.planes && oz_plane_elems(ldx, kTrsmOuter, kOzMaxDigits) <= c->trsm_sc.X.cap)
+    if (trsm_tc)
       trsm_lower_t_tc(la, c->L, NA, c->Xt, ldx, 0, c->trsm_sc);   // mixed mode: tensor-core updates
     else
       trsm_lower(la, c->L, NA, c->Xt, ldx, true, 0, c->trsm_tmp);
