@@ -1222,7 +1222,8 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
     }
     // matrices
     size_t n2 = (size_t)N * N, na2 = (size_t)NA * NA, big = (size_t)NA * n2;
-    c->S = dalloc<double>(n2); c->H = dalloc<double>(n2); c->Tk = dalloc<double>(n2); c->V = dalloc<double>(n2);
+    c->S = dalloc<double>(n2); c->H = dalloc<double>(n2);
+    if (!c->opt.pure) { c->Tk = dalloc<double>(n2); c->V = dalloc<double>(n2); }   // the lane kernels form h itself
     c->A = dalloc<double>(na2); c->L = dalloc<double>(na2); c->Linv = dalloc<double>(na2);
     c->npp = (long long)N * (N + 1) / 2;
     c->Bp = dalloc<double>((size_t)NA * c->npp); c->Yp = dalloc<double>((size_t)NA * c->npp);
