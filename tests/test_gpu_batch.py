@@ -59,6 +59,34 @@ def test_batch_step_without_new_geometry_and_errors():
 
 
 @pytest.mark.parametrize("precision", [0, 1])
+def test_batch_above_order_256(precision):
+    """Three members of 264 functions: their diagonalisations are cooperative launches with grid
+    barriers, on three streams at once, replayed from graphs from the second step on.  (The barriers'
+    waits are bounded: two that kept each other from the SMs would return an error.)  The SCFs stop at
+    max|e| < 1e-7: energies then differ by its square over the gap, forces by about 1e-7 over the gap
+    times derivative integrals of order one."""
+    R = _R()
+    mols = [W.water_n(11, seed) for seed in range(3)]
+    conv = dict(conv_e=1e-9, conv_diis=1e-7, max_iter=100)
+    ctxs = [R.Context(m, precision=precision, **conv) for m in mols]
+    E0, G0, _ = R.batch_step(ctxs, None, guess=5)
+    xs = [m.xyz + 0.002 * np.random.default_rng(i).standard_normal(m.xyz.shape) for i, m in enumerate(mols)]
+    for rep in range(3):
+        E, G, _ = R.batch_step(ctxs, xs if rep % 2 == 0 else [m.xyz for m in mols], guess=2)
+        if rep == 1:
+            assert np.abs(E - E0).max() <= 1e-8
+            assert max(np.abs(a - b).max() for a, b in zip(G, G0)) <= 1e-6
+    for c in ctxs:
+        c.close()
+    for m, x, e, g in zip(mols, xs, E, G):
+        c = R.Context(m, precision=precision, **conv)
+        c.update_geometry(x)
+        assert abs(c.scf(guess=5, outputs=False)["energy"] - e) <= 1e-8
+        assert np.abs(c.gradient() - g).max() <= 1e-6
+        c.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
 def test_cuda_graph_replay_matches_eager(precision):
     R = _R()
     mol = W.water_n(3, 0)

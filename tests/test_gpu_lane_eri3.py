@@ -53,7 +53,24 @@ def _conditioned(seed):
     return mol
 
 
+def _two_f_atoms():
+    """Two waters with one f shell each, 3.6 bohr apart: (f f| pairs over two atoms (overlap up to 0.18,
+    density 4e-3: their derivatives are 1e5 times the bound), lambda_min(S) = 0.059."""
+    mol = W.water_n(2, 7)
+    d = mol.xyz[3] - mol.xyz[0]
+    mol.xyz = mol.xyz.copy()
+    mol.xyz[3:] -= d * (1.0 - 3.6 / np.linalg.norm(d))
+    prim = {8: [(0, 0.35), (0, 1.9), (1, 0.5), (2, 0.9), (3, 0.5)], 1: [(0, 0.45)]}
+    aux = {8: [(0, 0.5), (0, 1.6), (0, 5.0), (1, 0.7), (1, 2.5), (2, 0.9), (2, 3.0), (3, 1.1), (4, 1.4)],
+           1: [(0, 0.5), (0, 1.8), (1, 0.9), (2, 1.2)]}
+    mol.primary = [W.Shell(a, l, [x], [1.0]) for a, z in enumerate(mol.Z) for l, x in prim[int(z)]]
+    mol.aux = [W.Shell(a, l, [x], [1.0]) for a, z in enumerate(mol.Z) for l, x in aux[int(z)]]
+    return mol
+
+
 def _case(name):
+    if name == "f on two atoms":
+        return _shuffled(_two_f_atoms(), 7)
     if name == "f and g conditioned":
         return _shuffled(_conditioned(5), 5)
     if name == "mixed contraction conditioned":
@@ -95,7 +112,7 @@ def test_metric_and_one_electron(name):
 
 
 @pytest.mark.parametrize("name", ["small shuffled", "f and g conditioned", "mixed contraction conditioned",
-                                  "middle distance"])
+                                  "middle distance", "f on two atoms"])
 def test_three_centre_derivatives(name):
     R = _R()
     mol = _case(name)
