@@ -1,5 +1,5 @@
 // Derivative contraction of the one-electron integrals for spherical bases:
-// 4 to 32 lanes per shell pair (build_one_tasks), which share out the nuclei and, for
+// 4 to 32 lanes per shell pair (one_lanes), which share out the nuclei and, for
 // overlap and kinetic energy, the Cartesian components.
 //
 // The derivative of nuclear attraction needs the weights w of the horizontal
@@ -11,7 +11,7 @@
 // (H2O)3 (666 pairs, 9 nuclei), 0.137 at (H2O)8, 1.08 at (H2O)10 in the larger basis; the
 // warp-cooperative kernel (a task per pair and nucleus, four recurrences each) takes
 // 0.105, 0.95 and 16.4 ms.  One water in the larger basis is the one case where it is
-// ahead, 0.182 against 0.199 ms: the serial chain of an (f f| pair.
+// ahead, 0.182 against 0.195 ms: the serial chain of an (f f| pair.
 #include <algorithm>
 
 #include "../../include/rihf.h"
@@ -166,20 +166,21 @@ __device__ __noinline__ void grad_one_tasks(const OneArgs& g, const LaneChunk& c
   }
 }
 
-// One block (warp) per chunk.
+// One warp a block.
 __global__ void __launch_bounds__(32, 8) lane_grad_one_kernel(const __grid_constant__ OneArgs g, const double* D,
                                                               const double* W, double* grad_one, double* grad_ovl) {
-  const LaneChunk ch = g.chunks[blockIdx.x];
+  LaneChunk ch;
+  if (!one_chunk(g, ch)) return;
   RIHF_ONE_CASES(grad_one_tasks, D, W, grad_one, grad_ovl)
 }
 
 }  // namespace
 
-void launch_lane_grad_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
-                          const double* axyz, const double* D, const double* W, double* grad_one, double* grad_ovl) {
+void launch_lane_grad_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int lanes, int natoms,
+                          const int* Z, const double* axyz, const double* D, const double* W, double* grad_one, double* grad_ovl) {
   if (t.nchunk <= 0) return;
-  lane_grad_one_kernel<<<(unsigned)t.nchunk, 32, 0, ic.stream>>>(one_args(ic, prim, t, natoms, Z, axyz), D, W, grad_one,
-                                                                 grad_ovl);
+  lane_grad_one_kernel<<<one_grid(t, lanes), 32, 0, ic.stream>>>(one_args(ic, prim, t, lanes, natoms, Z, axyz), D, W,
+                                                                 grad_one, grad_ovl);
   RIHF_LAUNCH_CHECK();
   if (ic.launches) *ic.launches += 1;
 }

@@ -10,7 +10,6 @@ struct Lane2Tasks {
   const int2* tasks = nullptr;
   const LaneChunk* chunks = nullptr;
   long long nchunk = 0;
-  int lanes = 1;   // lanes a task
 };
 
 // (P|Q): auxiliary shell pairs, the lower l first; cls = la | lc << 8.
@@ -22,14 +21,17 @@ void launch_lane_eri2(const IntegralCtx& ic, const DevShells& aux, const Lane2Ta
 void launch_lane_grad_eri2(const IntegralCtx& ic, const DevShells& aux, const Lane2Tasks& t, const KetTable* ket,
                            const double* Z, double* grad);
 
-// One-electron: primary shell pairs (a, b), la >= lb, 4 to 32 lanes each (the
-// nuclei shared out between them), the number returned; cls = la | lb << 4.
-int build_one_tasks(const std::vector<int>& l, int sms, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks);
+// One-electron: primary shell pairs (a, b), la >= lb, in chunks of at most kOneChunk;
+// cls = la | lb << 4.  A launch gives every pair 4 to 32 lanes, which share out the nuclei.
+constexpr int kOneChunk = 8;
+void build_one_tasks(const std::vector<int>& l, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks);
+// The lanes of a pair when `share` contexts launch at the same time.
+int one_lanes(int nshell, int natoms, int sms, int share);
 // S and h = T + V, both triangles.
-void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
+void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int lanes, int natoms, const int* Z,
                      const double* axyz, double* S, double* H);
 // grad_one += sum D d(T + V), grad_ovl += -sum W dS.
-void launch_lane_grad_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
-                          const double* axyz, const double* D, const double* W, double* grad_one, double* grad_ovl);
+void launch_lane_grad_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int lanes, int natoms,
+                          const int* Z, const double* axyz, const double* D, const double* W, double* grad_one, double* grad_ovl);
 
 }  // namespace rihf

@@ -1,6 +1,6 @@
 // One-electron integrals for spherical bases: 4 to 32 lanes per shell pair, which
 // share out the nuclei (the recursion of eri3_lane.cuh with a point-charge ket, i.e.
-// no ket steps; how many lanes: build_one_tasks).  Measured 0.077 ms at (H2O)8 (4656
+// no ket steps; how many lanes: one_lanes).  Measured 0.077 ms at (H2O)8 (4656
 // pairs, 24 nuclei), 0.38 ms at (H2O)10 in the larger basis; the warp-cooperative
 // kernel takes 0.39 and 3.1 ms.
 #include <algorithm>
@@ -101,9 +101,10 @@ __device__ __noinline__ void one_tasks(const OneArgs& g, const LaneChunk& ch, do
   store(S);
 }
 
-// One block (warp) per chunk.
+// One warp a block.
 __global__ void __launch_bounds__(32, 8) lane_one_kernel(const __grid_constant__ OneArgs g, double* S, double* H) {
-  const LaneChunk ch = g.chunks[blockIdx.x];
+  LaneChunk ch;
+  if (!one_chunk(g, ch)) return;
   RIHF_ONE_CASES(one_tasks, S, H)
 }
 }  // namespace
@@ -111,13 +112,22 @@ __global__ void __launch_bounds__(32, 8) lane_one_kernel(const __grid_constant__
 // The lanes of a pair: the most that leave at most 32 warps an SM.  Below that the
 // latency of one pair's chain over the nuclei is the time, and more lanes shorten it;
 // above, FP64 instructions count and the part of a pair that every lane repeats makes
-// more lanes dearer.  Derivatives with 4 / 8 / 16 / 32 lanes: (H2O)3, 666 pairs, 0.176 /
+// more lanes dearer (contexts of a batch launch beside each other, and each gets
+// its share: 16 of 3 to 6 waters take 0.7 ms longer in 102 when each fills the SMs by
+// itself).  No more than about two a nucleus (the components that the
+// derivative also shares out use the second): with three nuclei in the larger basis 32
+// lanes make the integrals 0.125 ms, 8 lanes 0.119.  Derivatives with 4 / 8 / 16 / 32 lanes: (H2O)3, 666 pairs, 0.176 /
 // 0.135 / 0.100 / 0.084 ms; (H2O)8, 4656 pairs, 0.268 / 0.176 / 0.143 / 0.139; (H2O)12,
 // 10440 pairs, 0.397 / 0.276 / 0.272 / 0.387.
-int build_one_tasks(const std::vector<int>& l, int sms, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks) {
-  const long long pairs = (long long)l.size() * (l.size() + 1) / 2;
-  int lanes = 32;
+int one_lanes(int nshell, int natoms, int sms, int share) {
+  const long long pairs = (long long)nshell * (nshell + 1) / 2 * share;
+  int lanes = 4;
+  while (lanes < 32 && lanes < 2 * natoms) lanes *= 2;
   while (lanes > 4 && pairs * lanes > 32LL * 32 * sms) lanes /= 2;
+  return lanes;
+}
+
+void build_one_tasks(const std::vector<int>& l, std::vector<int2>& tasks, std::vector<LaneChunk>& chunks) {
   std::vector<int> by_l[kMaxLPrim + 1];
   for (int i = 0; i < (int)l.size(); ++i) by_l[l[i]].push_back(i);
   tasks.clear();
@@ -129,16 +139,15 @@ int build_one_tasks(const std::vector<int>& l, int sms, std::vector<int2>& tasks
         for (int b : by_l[lb])
           if (la != lb || a >= b) tasks.push_back(make_int2(a, b));
       const long long n = (long long)tasks.size() - t0;
-      const int per = 32 / lanes;
-      for (long long i = 0; i < n; i += per) chunks.push_back({t0 + i, (int)std::min<long long>(per, n - i), la | lb << 4});
+      for (long long i = 0; i < n; i += kOneChunk)
+        chunks.push_back({t0 + i, (int)std::min<long long>(kOneChunk, n - i), la | lb << 4});
     }
-  return lanes;
 }
 
-void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
+void launch_lane_one(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int lanes, int natoms, const int* Z,
                      const double* axyz, double* S, double* H) {
   if (t.nchunk <= 0) return;
-  lane_one_kernel<<<(unsigned)t.nchunk, 32, 0, ic.stream>>>(one_args(ic, prim, t, natoms, Z, axyz), S, H);
+  lane_one_kernel<<<one_grid(t, lanes), 32, 0, ic.stream>>>(one_args(ic, prim, t, lanes, natoms, Z, axyz), S, H);
   RIHF_LAUNCH_CHECK();
   if (ic.launches) *ic.launches += 1;
 }

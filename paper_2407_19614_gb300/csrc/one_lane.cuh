@@ -90,10 +90,22 @@ struct OneArgs {
   const double* boys;
 };
 
-inline OneArgs one_args(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int natoms, const int* Z,
-                        const double* axyz) {
-  return OneArgs{prim, t.tasks, t.chunks, t.lanes, natoms, Z, axyz, ic.boys};
+inline OneArgs one_args(const IntegralCtx& ic, const DevShells& prim, const Lane2Tasks& t, int lanes, int natoms,
+                        const int* Z, const double* axyz) {
+  return OneArgs{prim, t.tasks, t.chunks, lanes, natoms, Z, axyz, ic.boys};
 }
+
+// The pairs of this warp: lanes / 4 blocks a chunk, 32 / lanes pairs each (a short
+// chunk's last blocks have none: false).
+__device__ __forceinline__ bool one_chunk(const OneArgs& g, LaneChunk& ch) {
+  const int blocks = g.lanes / (32 / kOneChunk), per = 32 / g.lanes;
+  ch = g.chunks[blockIdx.x / blocks];
+  const int at = (blockIdx.x % blocks) * per;
+  ch.task0 += at;
+  ch.n = min(per, ch.n - at);
+  return ch.n > 0;
+}
+inline unsigned one_grid(const Lane2Tasks& t, int lanes) { return (unsigned)(t.nchunk * (lanes / (32 / kOneChunk))); }
 
 // Runs f<la, lb>(g, ch, ...) for the class of chunk ch.
 #define RIHF_ONE_CASES(f, ...)                          \

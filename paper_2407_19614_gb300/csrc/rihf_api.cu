@@ -537,6 +537,7 @@ struct rihf_ctx {
   KetTable* d_ket = nullptr;
   Lane2Tasks lane_eri2, lane_one;    // (P|Q) and one-electron shell pairs, of the basis alone
   int2* d_tasks2 = nullptr;
+  int share = 1;                     // contexts that launch at the same time (a batch step)
   LaneChunk* d_chunks2 = nullptr;
   double* d_schwarz = nullptr;
   bool schwarz_ok = false;
@@ -867,7 +868,7 @@ static void compute_geometry(rihf_ctx* c, bool defer_eri3 = false) {
   DevShells P = c->prim(), X = c->aux();
   { TraceScope t(c->tracer, s, "one_electron_kernel (S,T,V)", 3.0 * N * N * 8, 1);
     if (c->opt.pure) {
-      launch_lane_one(ic, P, c->lane_one, c->natoms, c->d_Z, c->d_xyz, c->S, c->H);
+      launch_lane_one(ic, P, c->lane_one, one_lanes(c->hp.nshell, c->natoms, c->sms, c->share), c->natoms, c->d_Z, c->d_xyz, c->S, c->H);
     } else {
       launch_one_electron(ic, P, c->max_lp, c->natoms, c->d_Z, c->d_xyz, c->S, c->Tk, c->V);
       axpby(la, N * N, 1.0, c->Tk, 1.0, c->V, c->H);
@@ -1203,7 +1204,7 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       std::vector<int2> t2, t1;
       std::vector<LaneChunk> c2, c1;
       build_lane2_tasks(c->ha.l, c->ha.atom, t2, c2);
-      const int lanes = build_one_tasks(c->hp.l, c->sms, t1, c1);
+      build_one_tasks(c->hp.l, t1, c1);
       c->d_tasks2 = dalloc<int2>(t2.size() + t1.size());
       c->d_chunks2 = dalloc<LaneChunk>(c2.size() + c1.size());
       upload(c->d_tasks2, t2, s);
@@ -1212,7 +1213,7 @@ static rihf_ctx* setup_impl(int natoms, const int* Z, const double* xyz, int npr
       upload(c->d_chunks2 + c2.size(), c1, s);
       RIHF_CUDA(cudaStreamSynchronize(s));   // the host lists are temporaries
       c->lane_eri2 = {c->d_tasks2, c->d_chunks2, (long long)c2.size()};
-      c->lane_one = {c->d_tasks2 + t2.size(), c->d_chunks2 + c2.size(), (long long)c1.size(), lanes};
+      c->lane_one = {c->d_tasks2 + t2.size(), c->d_chunks2 + c2.size(), (long long)c1.size()};
     }
     refresh_tasks(c);
     {
@@ -2714,7 +2715,8 @@ static void gradient_launch(rihf_ctx* c, bool defer_eri3) {
   double* g_two = c->grad_parts + 9 * nat;
   { TraceScope t(c->tracer, s, "grad_one_electron_kernel", 0.0, 0);
     if (c->opt.pure)
-      launch_lane_grad_one(ic, c->prim(), c->lane_one, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl);
+      launch_lane_grad_one(ic, c->prim(), c->lane_one, one_lanes(c->hp.nshell, nat, c->sms, c->share), nat, c->d_Z,
+                           c->d_xyz, c->D, c->W, g_one, g_ovl);
     else
       launch_grad_one_electron(ic, c->prim(), c->max_lp, nat, c->d_Z, c->d_xyz, c->D, c->W, g_one, g_ovl); }
   if (!defer_eri3) {
@@ -2983,6 +2985,13 @@ int rihf_batch_step(int nmol, rihf_ctx* const* ctx, const double* const* xyz, in
   for (int i = 0; i < nmol; ++i) goff[i + 1] = goff[i] + 3 * (size_t)ctx[i]->natoms;
   std::vector<int> rc(nmol, RIHF_OK);
   std::vector<std::string> err(nmol);
+  struct Share {   // for the time of this call the members share the SMs
+    rihf_ctx* const* ctx;
+    int n;
+    Share(rihf_ctx* const* c, int m) : ctx(c), n(m) { set(m); }
+    ~Share() { set(1); }
+    void set(int v) { for (int i = 0; i < n; ++i) ctx[i]->share = v; }
+  } share(ctx, nmol);
   // The 3-centre integrals and the 3-centre derivative contraction, the
   // largest per-geometry launches, run as one launch per class group over all
   // molecules (launch_eri3_batch / launch_grad_eri3_batch: ragged task lists

@@ -1,7 +1,7 @@
 """The one-electron lane kernels at every number of lanes a pair, against the warp-cooperative ones.
 
 A basis of s and p shells is the same in Cartesian (x, y, z) and in spherical form (y, z, x), and the two
-forms run different kernels.  Clusters of 2, 10, 14 and 20 waters (10 such shells each) get 32, 16, 8 and 4
+forms run different kernels.  Clusters of 1, 4, 10, 14 and 20 waters (11 such shells each) get 8, 32, 16, 8 and 4
 lanes a pair on 152 SMs, with chunks that end inside a warp.  Integrals to the 1e-12 of the largest
 element of the other integral tests.  The forces come from two SCFs whose densities differ by about
 conv_diis over the gap (1e-9); a term of the gradient is that times its derivative integrals (below
@@ -15,7 +15,7 @@ from paper_2407_19614_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nwater", [2, 10, 14, 20])
+@pytest.mark.parametrize("nwater", [1, 4, 10, 14, 20])
 def test_lanes_against_warps(nwater):
     from paper_2407_19614_gb300 import rihf as R
     mol = W.water_n(nwater, 3)
