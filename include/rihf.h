@@ -112,7 +112,8 @@ int rihf_setup(int natoms, const int* Z, const double* xyz, int nprim_shells, co
 
 /* Moves the nuclei to xyz[natoms*3] (same atoms and basis) and recomputes every
    geometry-dependent quantity listed for rihf_setup.  Converged orbitals of the
-   previous geometry are kept as the default guess of the next rihf_scf. */
+   previous geometry are kept as the default guess of the next rihf_scf.
+   Errors: as rihf_setup. */
 int rihf_update_geometry(rihf_ctx* ctx, const double* xyz);
 
 /*
@@ -148,7 +149,9 @@ int rihf_update_geometry(rihf_ctx* ctx, const double* xyz);
  *          guess-4 SCF first trains the network on its own example
  *          (rihf_learn_config).
  *   energy (1), D (N*N), C (N*N), eps (N), iters (1): outputs; any may be NULL.
- * Returns NOT_CONVERGED (outputs filled from the last iterate) after max_iter.
+ * Returns NOT_CONVERGED (outputs filled from the last iterate) after max_iter,
+ * TIMEOUT when a bounded device wait ran out (no converged SCF afterwards;
+ * one in the guess history leaves the converged SCF and empties the history).
  */
 int rihf_scf(rihf_ctx* ctx, int guess, const double* C_guess, double* energy, double* D, double* C, double* eps,
              int* iters);
@@ -160,7 +163,7 @@ int rihf_scf(rihf_ctx* ctx, int guess, const double* C_guess, double* energy, do
  * with h^xi including the nuclear-attraction operator derivative.  The
  * derivative integrals are evaluated and contracted on the fly, never stored.
  *   grad: natoms*3 output, dE/dR (forces are its negative).
- * Errors: STATE if no converged SCF is available.
+ * Errors: STATE if no converged SCF is available, TIMEOUT.
  */
 int rihf_gradient(rihf_ctx* ctx, double* grad);
 

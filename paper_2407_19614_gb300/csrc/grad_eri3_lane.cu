@@ -11,7 +11,7 @@
 // so only (a b-1| runs a recurrence on the integrals.
 //
 // Bound by the FP64 pipe: 4.7e8 FP64 instructions a lane set for (H2O)8 (0.78 ms
-// at its rate), 9.5e9 for (H2O)10 in the larger basis (15.9 ms).  Measured 1.40
+// at its rate), 9.5e9 for (H2O)10 in the larger basis (15.9 ms).  Measured 1.30
 // and 19.5 ms; the warp-cooperative kernel with its four recurrences
 // (grad_integrals.cu) takes 11.2 and 251 ms.
 #include <algorithm>

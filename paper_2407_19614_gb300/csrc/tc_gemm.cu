@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int col0 = (warp >> 2) * ncol;
     const uint32_t t_row = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
     // one thread polls, the other drain threads wait on a hardware named
-    // barrier (spinning 256 threads would compete with the copy and MMA
+    // barrier (spinning 512 threads would compete with the copy and MMA
     // threads for issue slots and for the barrier unit); the poller is lane 0
     // of warp 2, on a scheduler that neither the MMA nor the copy warp uses
     int nwait = 0;
