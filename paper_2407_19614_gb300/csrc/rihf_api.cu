@@ -2525,7 +2525,7 @@ int rihf_scf(rihf_ctx* c, int guess, const double* C_guess, double* energy, doub
   if (tc_flag) late();
   if (conv) {
     learn_and_push_history(c);
-    inject_late(c, RIHF_WAIT_HISTORY);
+    if (c->hist_lowdin) inject_late(c, RIHF_WAIT_HISTORY);   // (without Loewdin factors nothing waits)
     if (c->hist_lowdin && late_take(c)) {   // the SCF's own results stand
       c->nhist = 0;
       c->lowdin_serial = -1;

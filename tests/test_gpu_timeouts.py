@@ -37,6 +37,16 @@ def test_expired_wait_is_reported(point, precision):
     ctx.close()
 
 
+def test_a_point_that_is_not_reached_raises_nothing():
+    from paper_2407_19614_gb300 import rihf as R
+    mol = W.water_monomer(1)
+    ctx = R.Context(mol)
+    ctx.inject_timeout("HISTORY")   # guess 0 keeps no Loewdin history
+    ctx.scf(guess=0, outputs=False)
+    ctx.gradient()
+    ctx.close()
+
+
 def test_batch_reports_the_member():
     from paper_2407_19614_gb300 import rihf as R
     mols = [W.water_n(n, n) for n in (1, 2)]
